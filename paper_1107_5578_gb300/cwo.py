@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -34,6 +35,7 @@ DEFAULT_PITCH = 10e-6
 
 _lock = threading.Lock()
 _lib = None
+_torch = None
 
 
 class Shift(ctypes.Structure):
@@ -63,6 +65,17 @@ class Item(ctypes.Structure):
                 ("dy", ctypes.c_double), ("type", ctypes.c_int), ("flags", ctypes.c_uint)]
 
 
+# the same record for struct.pack_into: filling one per item takes a third of the time of building
+# ctypes structures one by one
+_ITEM = struct.Struct("@ddddiI")
+assert _ITEM.size == ctypes.sizeof(Item)
+
+
+def _int32(v: int) -> int:
+    """v wrapped to 32 bits, as a C int field takes it"""
+    return (v + (1 << 31)) % (1 << 32) - (1 << 31)
+
+
 class CwoError(RuntimeError):
     def __init__(self, status: int, where: str, message: str):
         self.status = status
@@ -72,6 +85,8 @@ class CwoError(RuntimeError):
 def lib() -> ctypes.CDLL:
     """Load the shared library (built by ``__graft_entry__.build()``); raise if it is missing."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -138,14 +153,27 @@ def device_bytes(nx: int, ny: int, batch: int = 1) -> int:
     return int(out.value)
 
 
-def _stream_handle(stream) -> ctypes.c_void_p:
-    import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(int(s.cuda_stream))
+def _load_torch():
+    """torch, imported by the first call that touches a tensor (the host-only entry points do not
+    need it) and kept: an import statement in every call costs about a microsecond."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
+def _stream_handle(stream) -> int:
+    """cudaStream_t of ``stream`` (None: the current device's current stream, read as a plain
+    integer: building a torch.cuda.Stream object costs several microseconds)."""
+    if stream is None:
+        torch = _torch or _load_torch()
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return int(stream.cuda_stream)
 
 
 def _check_field(t, nx: int, ny: int, name: str, batch: int | None = None):
-    import torch
+    torch = _torch or _load_torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != torch.complex64:
@@ -154,14 +182,15 @@ def _check_field(t, nx: int, ny: int, name: str, batch: int | None = None):
         raise ValueError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if tuple(t.shape[-2:]) != (ny, nx):
-        raise ValueError(f"{name} has shape {tuple(t.shape)}, expected [..., {ny}, {nx}]")
+    s = t.shape
+    if len(s) < 2 or s[-1] != nx or s[-2] != ny:
+        raise ValueError(f"{name} has shape {tuple(s)}, expected [..., {ny}, {nx}]")
     if batch is not None and t.numel() != batch * nx * ny:
         raise ValueError(f"{name} holds {t.numel() // (nx * ny)} fields, expected {batch}")
 
 
 def _check_real(t, nx: int, ny: int, name: str, batch: int):
-    import torch
+    torch = _torch or _load_torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != torch.float32:
@@ -259,26 +288,30 @@ class Plan:
         return int(lib().cwo_launches_per_call(self.handle))
 
     def _out(self, x, batch_shape):
-        import torch
+        torch = _torch or _load_torch()
         return torch.empty((*batch_shape, self.ny, self.nx), dtype=torch.complex64, device=x.device)
+
+    def _result(self, x, out, batch_shape, batch):
+        """``out`` once checked, or a new output (which needs no check)"""
+        if out is None:
+            return self._out(x, batch_shape)
+        _check_field(out, self.nx, self.ny, "output", batch)
+        return out
+
+    def _one(self, fn, name, x, out, stream):
+        _check_field(x, self.nx, self.ny, "input", 1)
+        out = self._result(x, out, x.shape[:-2], 1)
+        st = fn(self.handle, x.data_ptr(), out.data_ptr(), _stream_handle(stream))
+        if st != OK:
+            check(st, name)
+        return out
 
     def propagate(self, x, out=None, stream=None):
         """One field [Ny][Nx] (complex64, CUDA) -> propagated field."""
-        _check_field(x, self.nx, self.ny, "input", 1)
-        out = self._out(x, x.shape[:-2]) if out is None else out
-        _check_field(out, self.nx, self.ny, "output", 1)
-        check(lib().cwo_propagate(self.handle, ctypes.c_void_p(x.data_ptr()),
-                                  ctypes.c_void_p(out.data_ptr()), _stream_handle(stream)), "cwo_propagate")
-        return out
+        return self._one(lib().cwo_propagate, "cwo_propagate", x, out, stream)
 
     def adjoint(self, x, out=None, stream=None):
-        _check_field(x, self.nx, self.ny, "input", 1)
-        out = self._out(x, x.shape[:-2]) if out is None else out
-        _check_field(out, self.nx, self.ny, "output", 1)
-        check(lib().cwo_propagate_adjoint(self.handle, ctypes.c_void_p(x.data_ptr()),
-                                          ctypes.c_void_p(out.data_ptr()), _stream_handle(stream)),
-              "cwo_propagate_adjoint")
-        return out
+        return self._one(lib().cwo_propagate_adjoint, "cwo_propagate_adjoint", x, out, stream)
 
     def propagate_batch(self, x, z=None, out=None, stream=None, adjoint=False):
         """Batch [B][Ny][Nx] -> [B][Ny][Nx].  ``z``: None (plan z) or B distances (host floats)."""
@@ -293,25 +326,25 @@ class Plan:
         _check_field(x, self.nx, self.ny, "input", b)
         if len(items) != b:
             raise ValueError(f"{len(items)} items for {b} fields")
-        arr = (Item * b)()
+        buf = bytearray(b * ctypes.sizeof(Item))
         for k, it in enumerate(items):
             if isinstance(it, Item):
-                arr[k] = it
+                buf[k * _ITEM.size:(k + 1) * _ITEM.size] = bytes(it)
             else:
-                arr[k] = Item(float(it["z"]), float(it["wavelength"]), float(it["dx"]),
-                              float(it.get("dy", it["dx"])), int(it["type"]), int(it.get("flags", 0)))
-        out = self._out(x, (b,)) if out is None else out
-        _check_field(out, self.nx, self.ny, "output", b)
-        check(lib().cwo_propagate_items(self.handle, ctypes.c_void_p(x.data_ptr()), self.nx * self.ny,
-                                        ctypes.c_void_p(out.data_ptr()), b, arr, _stream_handle(stream)),
-              "cwo_propagate_items")
+                _ITEM.pack_into(buf, k * _ITEM.size, float(it["z"]), float(it["wavelength"]), float(it["dx"]),
+                                float(it.get("dy", it["dx"])), _int32(int(it["type"])),
+                                int(it.get("flags", 0)) & 0xFFFFFFFF)
+        arr = (Item * b).from_buffer(buf)
+        out = self._result(x, out, (b,), b)
+        check(lib().cwo_propagate_items(self.handle, x.data_ptr(), self.nx * self.ny, out.data_ptr(), b, arr,
+                                        _stream_handle(stream)), "cwo_propagate_items")
         return out
 
     def propagate_epilogue(self, x, epilogue, amplitude=None, out=None, adjoint=False, stream=None):
         """Batch [B][Ny][Nx] (or one field) propagated (adjoint: by conj(H)) with an output
         epilogue: EPI_PHASE (unit amplitude), EPI_AMPLITUDE (amplitude * phase; ``amplitude`` a
         float32 tensor shaped like x) or EPI_INTENSITY (returns |u|^2 as float32)."""
-        import torch
+        torch = _torch or _load_torch()
         b = x.shape[0] if x.dim() == 3 else 1
         _check_field(x, self.nx, self.ny, "input", b)
         inten = None
@@ -337,7 +370,7 @@ class Plan:
         """Gerchberg-Saxton kinoform iteration in place on ``field`` ([B][Ny][Nx] or one field;
         in: amplitude * initial phase, out: the kinoform).  Returns the reconstructed intensity
         (float32, like ``amplitude``) or None."""
-        import torch
+        torch = _torch or _load_torch()
         b = field.shape[0] if field.dim() == 3 else 1
         _check_field(field, self.nx, self.ny, "field", b)
         _check_real(amplitude, self.nx, self.ny, "amplitude", b)
@@ -353,17 +386,16 @@ class Plan:
         return self._batch(x, 0, len(zs), zs, out, stream, False)
 
     def _batch(self, x, stride, b, z, out, stream, adjoint):
-        out = self._out(x, (b,)) if out is None else out
-        _check_field(out, self.nx, self.ny, "output", b)
+        out = self._result(x, out, (b,), b)
         zp = None
         if z is not None:
             if len(z) != b:
                 raise ValueError(f"{len(z)} distances for {b} items")
-            zarr = (ctypes.c_double * b)(*[float(v) for v in z])
-            zp = ctypes.cast(zarr, ctypes.POINTER(ctypes.c_double))
+            zp = (ctypes.c_double * b)(*map(float, z))
         fn = lib().cwo_propagate_adjoint_batch if adjoint else lib().cwo_propagate_batch
-        check(fn(self.handle, ctypes.c_void_p(x.data_ptr()), int(stride), ctypes.c_void_p(out.data_ptr()),
-                 int(b), zp, _stream_handle(stream)), fn.__name__)
+        st = fn(self.handle, x.data_ptr(), int(stride), out.data_ptr(), int(b), zp, _stream_handle(stream))
+        if st != OK:
+            check(st, fn.__name__)
         return out
 
 
