@@ -14,7 +14,10 @@ LIB = os.path.join(HERE, "libcwo_gb300.so")
 
 CUDA_HOME = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CU_SOURCES = ["cwo_rows.cu", "cwo_rows_inv_a.cu", "cwo_rows_inv_b.cu", "cwo_rows_turn.cu", "cwo_cols.cu", "cwo_cols_a.cu", "cwo_cols_b.cu", "cwo_cols_c.cu", "cwo_noalloc.cu", "cwo_fourier.cu", "cwo_lines.cu", "cwo_copy.cu", "cwo_calib.cu"]
+CU_SOURCES = ["cwo_rows.cu", "cwo_rows_inv_a.cu", "cwo_rows_inv_b.cu", "cwo_rows_turn.cu", "cwo_cols.cu", "cwo_cols_a.cu", "cwo_cols_b.cu", "cwo_cols_c.cu", "cwo_noalloc.cu", "cwo_fourier.cu", "cwo_lines.cu", "cwo_copy.cu", "cwo_itables.cu", "cwo_calib.cu"]
+# the FP64 table entries are computed on the host and on the device: neither contracts a multiply and
+# an add, so that both give the same bits
+FILE_FLAGS = {"cwo_itables.cu": ["-fmad=false"], "cwo_tables.cpp": ["-ffp-contract=off"]}
 CPP_SOURCES = ["cwo_plan.cpp", "cwo_tables.cpp", "cwo_emu.cpp", "cwo_serve.cpp"]
 
 
@@ -36,12 +39,12 @@ def _compile(src: str, verbose: bool) -> str:
     obj = os.path.join(OUT_DIR, os.path.basename(src) + ".o")
     inc = ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
     if src.endswith(".cu"):
-        cmd = [_nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
+        cmd = [_nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", *FILE_FLAGS.get(src, []),
                *inc, *os.environ.get("CWO_EXTRA_NVCC_FLAGS", "").split(), "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
     else:
-        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", *inc, "-I", os.path.join(CUDA_HOME, "include"),
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", *FILE_FLAGS.get(src, []), *inc, "-I", os.path.join(CUDA_HOME, "include"),
                "-c", os.path.join(CSRC, src), "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:

@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "cwo_tables.h"
+
 namespace cwo {
 
 enum HMode : int {
@@ -24,6 +26,23 @@ struct ItemParams {
     float kf;                 // K = z / lambda (series / closed-form tail)
     double K, sx, sy;         // FP64 per-element arm
 };
+
+// The items of one launch of k_asm_tables (cwo_itables.cu); tables: this item has angular-spectrum
+// tables (otherwise only its parameters are stored).  The list travels in the launch's parameters.
+struct AsmItem {
+    host::AsmAxis x, y;
+    ItemParams prm;
+    int tables;
+};
+constexpr int kAsmItems = 24;   // below the 4 KB that any launch can carry
+struct AsmItemList {
+    AsmItem item[kAsmItems];
+};
+static_assert(sizeof(AsmItemList) <= 3968, "launch parameters");
+// tables of `items` <= kAsmItems items into tx [items][px], ty [items][py] (axis index order, signed bins
+// kbx, kby), and, where given, their parameters into prm and z / lambda into kf
+cudaError_t launch_asm_tables(const AsmItemList& list, int items, const int* kbx, const int* kby, int px, int py, float4* tx,
+                              float4* ty, ItemParams* prm, float* kf, cudaStream_t st);
 
 // Transfer-function description for the column pass.  Per-axis tables are indexed by the axis
 // index idx = e * T + t (register e of thread t in the last forward stage, i.e. DIF position

@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -340,14 +341,13 @@ cwo_status ensure_ztables(cwo_plan* p, int items) {
     if (p->type == CWO_ANGULAR) {
         if ((st = dev_alloc(&p->zax, nx4, "per-item x tables")) || (st = dev_alloc(&p->zay, ny4, "per-item y tables")) ||
             (st = dev_alloc(&p->zkf, (size_t)items, "per-item K")))
-            return st;
-        zbytes = (nx4 + ny4) * sizeof(float4) + items * sizeof(float);
+            return st;   // filled on the device: no staging
     } else {
         if ((st = dev_alloc(&p->zhx, nx4, "per-item x tables")) || (st = dev_alloc(&p->zhy, ny4, "per-item y tables")))
             return st;
         zbytes = (nx4 + ny4) * sizeof(float2);
     }
-    if ((st = staging_alloc(p->zstage, zbytes))) return st;
+    if (zbytes && (st = staging_alloc(p->zstage, zbytes))) return st;
     p->zcap = items;
     return CWO_OK;
 }
@@ -394,6 +394,35 @@ cwo::HParams base_hparams(const cwo_plan* p, const double* zs, int batch) {
     }
     hp.ax = p->ax; hp.ay = p->ay; hp.kf = p->kf; hp.hx = p->hx; hp.hy = p->hy;
     return hp;
+}
+
+// Angular-spectrum tables of `items` parameter sets (params(i)) on the device, kAsmItems a launch;
+// fresnel(i) (null: none): item i has no such tables, only parameters.
+struct AsmParams { double z, lambda, dx, dy; };
+template <class Params>
+cwo_status asm_tables(const cwo_plan* p, int items, const Params& params, const bool* fresnel, float4* tx, float4* ty,
+                      cwo::ItemParams* prm, float* kf, cudaStream_t s) {
+    cwo::AsmItemList list;
+    for (int i0 = 0; i0 < items; i0 += cwo::kAsmItems) {
+        const int n = std::min(items - i0, cwo::kAsmItems);
+        for (int i = 0; i < n; ++i) {
+            const AsmParams q = params(i0 + i);
+            cwo::AsmItem& it = list.item[i];
+            it.tables = !(fresnel && fresnel[i0 + i]);
+            it.x = asm_axis(p->px, q.dx, q.lambda, q.z, true);
+            it.y = asm_axis(p->py, q.dy, q.lambda, q.z, false);
+            const int tm = asm_tail_mode(p->px, p->py, q.dx, q.dy, q.lambda, q.z);
+            it.prm.mode = !it.tables ? cwo::HMODE_FRESNEL : tm == 0 ? cwo::HMODE_ASM_POLY : tm == 1 ? cwo::HMODE_ASM_EXACT : cwo::HMODE_ASM_FP64;
+            it.prm.kf = (float)(q.z / q.lambda);
+            it.prm.K = q.z / q.lambda;
+            it.prm.sx = q.lambda * q.lambda / ((double)p->px * q.dx * (double)p->px * q.dx);
+            it.prm.sy = q.lambda * q.lambda / ((double)p->py * q.dy * (double)p->py * q.dy);
+        }
+        const cudaError_t e = cwo::launch_asm_tables(list, n, p->kb_x, p->kb_y, p->px, p->py, tx + (size_t)i0 * p->px,
+                                                     ty + (size_t)i0 * p->py, prm ? prm + i0 : nullptr, kf ? kf + i0 : nullptr, s);
+        if (e != cudaSuccess) return cuda_fail(e, "table launch");
+    }
+    return CWO_OK;
 }
 
 // prevalidated: the caller (one API call that propagates the same buffers repeatedly) has
@@ -481,23 +510,15 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
     } else if (zs && !per_item_k) {
         p->zs_cached.clear();
         if ((st = ensure_ztables(p, batch))) return st;
-        char* hb = nullptr;
-        int zslot = 0;
-        if ((st = staging_acquire(p->zstage, &hb, &zslot))) return st;
         if (p->type == CWO_ANGULAR) {
-            float4* hax = (float4*)hb;
-            float4* hay = hax + (size_t)batch * p->px;
-            float* hkf = (float*)(hay + (size_t)batch * p->py);
-            for (int i = 0; i < batch; ++i)
-                host_h_tables(p, zs[i], hax + (size_t)i * p->px, hay + (size_t)i * p->py, nullptr, nullptr, hkf + i);
-            cudaError_t e;
-            if ((e = cudaMemcpyAsync(p->zax, hax, (size_t)batch * p->px * sizeof(float4), cudaMemcpyHostToDevice, s)) ||
-                (e = cudaMemcpyAsync(p->zay, hay, (size_t)batch * p->py * sizeof(float4), cudaMemcpyHostToDevice, s)) ||
-                (e = cudaMemcpyAsync(p->zkf, hkf, (size_t)batch * sizeof(float), cudaMemcpyHostToDevice, s)))
-                return cuda_fail(e, "table upload");
+            auto params = [&](int i) { return AsmParams{zs[i], p->lambda, p->dx, p->dy}; };
+            if ((st = asm_tables(p, batch, params, nullptr, p->zax, p->zay, nullptr, p->zkf, s))) return st;
             hp.ax = p->zax; hp.ay = p->zay; hp.kf = p->zkf;
             hp.x_item_stride = p->px; hp.y_item_stride = p->py; hp.kf_item_stride = 1;
         } else {
+            char* hb = nullptr;
+            int zslot = 0;
+            if ((st = staging_acquire(p->zstage, &hb, &zslot))) return st;
             float2* hhx = (float2*)hb;
             float2* hhy = hhx + (size_t)batch * p->px;
             for (int i = 0; i < batch; ++i)
@@ -508,8 +529,8 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
                 return cuda_fail(e, "table upload");
             hp.hx = p->zhx; hp.hy = p->zhy;
             hp.x_item_stride = p->px; hp.y_item_stride = p->py;
+            if ((st = staging_release_after(p->zstage, zslot, s))) return st;
         }
-        if ((st = staging_release_after(p->zstage, zslot, s))) return st;
         p->zs_cached.assign(zs, zs + batch);
     } else {
         hp.ax = p->ax; hp.ay = p->ay; hp.kf = p->kf; hp.hx = p->hx; hp.hy = p->hy;
@@ -635,38 +656,25 @@ cwo_status ensure_itables(cwo_plan* p, int items) {
     if ((st = dev_alloc(&p->ix, nx4, "item x tables")) || (st = dev_alloc(&p->iy, ny4, "item y tables")) ||
         (st = dev_alloc(&p->iprm, (size_t)items, "item parameters")))
         return st;
-    if ((st = staging_alloc(p->istage, (nx4 + ny4) * sizeof(float4) + (size_t)items * sizeof(cwo::ItemParams)))) return st;
+    if ((st = staging_alloc(p->istage, (nx4 + ny4) * sizeof(float4)))) return st;
     p->icap = items;
     return CWO_OK;
 }
 
-// the tables and scalars of one item of a mixed batch.  lines: a Fresnel item that takes the two
-// separable line passes, whose tables are stored as P complex64 values at the start of the item's
-// rows (the line pass's layout); otherwise float4 rows (the column pass's layout).
-void item_tables(const cwo_plan* p, const cwo_item& it, float4* xt, float4* yt, cwo::ItemParams* prm, bool lines) {
-    const AxisGeo gx(p->px), gy(p->py);
-    if (it.type == CWO_ANGULAR) {
-        asm_axis_table(gx, it.dx, it.lambda, it.z, true, xt);
-        asm_axis_table(gy, it.dy, it.lambda, it.z, false, yt);
-        const int tm = asm_tail_mode(p->px, p->py, it.dx, it.dy, it.lambda, it.z);
-        prm->mode = tm == 0 ? cwo::HMODE_ASM_POLY : tm == 1 ? cwo::HMODE_ASM_EXACT : cwo::HMODE_ASM_FP64;
+// the tables of one Fresnel item of a mixed batch.  lines: an item that takes the two separable line
+// passes, whose tables are stored as P complex64 values at the start of the item's rows (the line
+// pass's layout); otherwise float4 rows (the column pass's layout).
+void fresnel_item_tables(const cwo_plan* p, const cwo_item& it, float4* xt, float4* yt, bool lines) {
+    std::vector<float2> hx(p->px), hy(p->py);
+    make_h_tables(p->px, p->py, it.dx, it.dy, it.lambda, it.z, true, (it.flags & CWO_FLAG_LITERAL_SCALE) != 0,
+                  nullptr, nullptr, hx.data(), hy.data(), nullptr);
+    if (lines) {
+        std::copy(hx.begin(), hx.end(), (float2*)xt);
+        std::copy(hy.begin(), hy.end(), (float2*)yt);
     } else {
-        std::vector<float2> hx(p->px), hy(p->py);
-        make_h_tables(p->px, p->py, it.dx, it.dy, it.lambda, it.z, true, (it.flags & CWO_FLAG_LITERAL_SCALE) != 0,
-                      nullptr, nullptr, hx.data(), hy.data(), nullptr);
-        if (lines) {
-            std::copy(hx.begin(), hx.end(), (float2*)xt);
-            std::copy(hy.begin(), hy.end(), (float2*)yt);
-        } else {
-            for (int i = 0; i < p->px; ++i) xt[i] = make_float4(hx[i].x, hx[i].y, 0.f, 0.f);
-            for (int i = 0; i < p->py; ++i) yt[i] = make_float4(hy[i].x, hy[i].y, 0.f, 0.f);
-        }
-        prm->mode = cwo::HMODE_FRESNEL;
+        for (int i = 0; i < p->px; ++i) xt[i] = make_float4(hx[i].x, hx[i].y, 0.f, 0.f);
+        for (int i = 0; i < p->py; ++i) yt[i] = make_float4(hy[i].x, hy[i].y, 0.f, 0.f);
     }
-    prm->kf = (float)(it.z / it.lambda);
-    prm->K = it.z / it.lambda;
-    prm->sx = it.lambda * it.lambda / ((double)p->px * it.dx * (double)p->px * it.dx);
-    prm->sy = it.lambda * it.lambda / ((double)p->py * it.dy * (double)p->py * it.dy);
 }
 
 cwo_status run_items(cwo_plan* p, const void* in, long long in_stride, void* out, int batch, const cwo_item* items,
@@ -689,41 +697,67 @@ cwo_status run_items(cwo_plan* p, const void* in, long long in_stride, void* out
     if ((st = check_device_range(in, (size_t)(batch - 1) * in_stride * sizeof(float2) + fb, p->device, "input"))) return st;
     if ((st = check_device_range(out, (size_t)batch * fb, p->device, "output"))) return st;
     if ((st = ensure_scratch(p, batch)) || (st = ensure_itables(p, batch))) return st;
-    char* hb = nullptr;
-    int islot = 0;
-    if ((st = staging_acquire(p->istage, &hb, &islot))) return st;
-    float4* hx = (float4*)hb;
-    float4* hy = hx + (size_t)batch * p->px;
-    cwo::ItemParams* hp_items = (cwo::ItemParams*)(hy + (size_t)batch * p->py);
-    // per-item FP64 tables, items spread over host threads when there is enough work
-    const size_t work = (size_t)batch * (p->px + p->py);
-    const int nthreads = (int)std::min<size_t>((size_t)std::max(1u, std::thread::hardware_concurrency()),
-                                               std::min<size_t>((size_t)batch, work / 8192 + 1));
     // Route: a Fresnel convolution item takes the two separable line passes (32 N^2 bytes, as a
     // Fresnel plan does) where the output allows their TMA stores, every other item the three
     // passes; each contiguous run of one route is one sub-batch.  An item's result therefore does
     // not depend on the other items of the batch.
     const bool lines_ok = (uintptr_t)out % 16 == 0;
     auto lines = [&](int i) { return lines_ok && items[i].type == CWO_FRESNEL_CONV; };
-    auto worker = [&](int w) {
-        for (int i = w; i < batch; i += nthreads)
-            item_tables(p, items[i], hx + (size_t)i * p->px, hy + (size_t)i * p->py, hp_items + i, lines(i));
-    };
-    if (nthreads <= 1) {
-        worker(0);
-    } else {
-        std::vector<std::thread> pool;
-        for (int w = 1; w < nthreads; ++w) pool.emplace_back(worker, w);
-        worker(0);
-        for (auto& th : pool) th.join();
-    }
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e;
-    if ((e = cudaMemcpyAsync(p->ix, hx, (size_t)batch * p->px * sizeof(float4), cudaMemcpyHostToDevice, s)) ||
-        (e = cudaMemcpyAsync(p->iy, hy, (size_t)batch * p->py * sizeof(float4), cudaMemcpyHostToDevice, s)) ||
-        (e = cudaMemcpyAsync(p->iprm, hp_items, (size_t)batch * sizeof(cwo::ItemParams), cudaMemcpyHostToDevice, s)))
-        return cuda_fail(e, "item table upload");
-    if ((st = staging_release_after(p->istage, islot, s))) return st;
+    // angular-spectrum tables and every item's parameters on the device
+    std::unique_ptr<bool[]> fresnel(new (std::nothrow) bool[batch]);
+    if (!fresnel) return fail(CWO_ERR_OOM, "host allocation failed");
+    int nf = 0;
+    for (int i = 0; i < batch; ++i) nf += (fresnel[i] = items[i].type == CWO_FRESNEL_CONV);
+    if (nf < batch || !lines_ok) {
+        auto params = [&](int i) { return AsmParams{items[i].z, items[i].lambda, items[i].dx, items[i].dy}; };
+        if ((st = asm_tables(p, batch, params, fresnel.get(), p->ix, p->iy, p->iprm, nullptr, s))) return st;
+    }
+    // Fresnel tables (an FP64 transform each) on the host, on threads when there is enough work, and
+    // one upload per contiguous run of Fresnel items.  Called ahead of the first run that has one:
+    // by then the angular-spectrum runs before it are under way on the GPU.
+    bool fresnel_ready = nf == 0;
+    auto fresnel_tables = [&]() -> cwo_status {
+        fresnel_ready = true;
+        char* hb = nullptr;
+        int islot = 0;
+        if ((st = staging_acquire(p->istage, &hb, &islot))) return st;
+        float4* hx = (float4*)hb;
+        float4* hy = hx + (size_t)nf * p->px;
+        const size_t work = (size_t)nf * (p->px + p->py);
+        const int nthreads = (int)std::min<size_t>((size_t)std::max(1u, std::thread::hardware_concurrency()),
+                                                   std::min<size_t>((size_t)nf, work / 8192 + 1));
+        auto worker = [&](int w) {
+            for (int i = 0, f = 0; i < batch; ++i) {
+                if (!fresnel[i]) continue;
+                if (f % nthreads == w)
+                    fresnel_item_tables(p, items[i], hx + (size_t)f * p->px, hy + (size_t)f * p->py, lines(i));
+                ++f;
+            }
+        };
+        if (nthreads <= 1) {
+            worker(0);
+        } else {
+            std::vector<std::thread> pool;
+            for (int w = 1; w < nthreads; ++w) pool.emplace_back(worker, w);
+            worker(0);
+            for (auto& th : pool) th.join();
+        }
+        for (int i0 = 0, f = 0; i0 < batch;) {
+            int i1 = i0 + 1;
+            while (i1 < batch && fresnel[i1] == fresnel[i0]) ++i1;
+            const size_t n = (size_t)(i1 - i0);
+            if (fresnel[i0]) {
+                if ((e = cudaMemcpyAsync(p->ix + (size_t)i0 * p->px, hx + (size_t)f * p->px, n * p->px * sizeof(float4), cudaMemcpyHostToDevice, s)) ||
+                    (e = cudaMemcpyAsync(p->iy + (size_t)i0 * p->py, hy + (size_t)f * p->py, n * p->py * sizeof(float4), cudaMemcpyHostToDevice, s)))
+                    return cuda_fail(e, "item table upload");
+                f += (int)n;
+            }
+            i0 = i1;
+        }
+        return staging_release_after(p->istage, islot, s);
+    };
 
     const long long wstride = (long long)p->ny * p->px;
     const float scale = (float)(1.0 / ((double)p->px * (double)p->py));
@@ -737,6 +771,9 @@ cwo_status run_items(cwo_plan* p, const void* in, long long in_stride, void* out
         while (i1 < batch && lines(i1) == lines(i0)) ++i1;
         const int n = i1 - i0;
         const bool last = i1 == batch;
+        if (!fresnel_ready && std::find(fresnel.get() + i0, fresnel.get() + i1, true) != fresnel.get() + i1 &&
+            (st = fresnel_tables()))
+            return st;
         if (lines(i0)) {
             CUtensorMap omap;
             if ((e = cwo::make_intermediate_map(&omap, fout + i0 * field, p->nx, p->ny, n, cwo::line_block_rows(p->py))))

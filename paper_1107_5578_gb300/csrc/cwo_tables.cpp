@@ -250,25 +250,25 @@ cd fresnel_coeff(double dx, double dy, double lambda, double z, bool literal_sca
     return c;
 }
 
-void asm_axis_table(const AxisGeo& g, double pitch, double lambda, double z, bool is_x, float4* out) {
+AsmAxis asm_axis(int P, double pitch, double lambda, double z, bool is_x) {
     const double K = z / lambda;
-    const double c0 = is_x ? frac01(K) : 0.0;
-    const double sgn = (is_x && K < 0) ? -1.0 : 1.0;
-    const double rt = std::sqrt(std::fabs(K)) * 0.5;
-    const double Pd = (double)g.P * pitch;
-    const double c1 = z * lambda / (2.0 * Pd * Pd);                              // K a / 2   per kt^2
-    const double c2 = z * lambda * lambda * lambda / (8.0 * Pd * Pd * Pd * Pd);  // K a^2 / 8 per kt^4
+    const double Pd = (double)P * pitch;
+    AsmAxis A;
+    A.lam2 = lambda * lambda;
+    A.pd2 = Pd * Pd;
+    A.c1 = z * lambda / (2.0 * Pd * Pd);
+    A.c2 = z * lambda * lambda * lambda / (8.0 * Pd * Pd * Pd * Pd);
+    A.c0 = is_x ? frac01(K) : 0.0;
+    A.su = (is_x && K < 0 ? -1.0 : 1.0) * (std::sqrt(std::fabs(K)) * 0.5);
+    return A;
+}
+
+void asm_axis_table(const AxisGeo& g, double pitch, double lambda, double z, bool is_x, float4* out) {
+    const AsmAxis A = asm_axis(g.P, pitch, lambda, z, is_x);
     // every entry depends on kt^2 only: evaluate |kt| = 0 .. P/2 once, store at both indices
     const AxisCache& c = axis_cache(g.P);
     for (int k = 0; k <= g.P / 2; ++k) {
-        const double kt = (double)k;
-        const double k2 = kt * kt;
-        const double a = lambda * lambda * k2 / (Pd * Pd);
-        const double W = frac01(frac01(c1 * k2) + frac01(c2 * k2 * k2)) - c0;
-        const double u = sgn * rt * a;
-        const float uh = (float)u;
-        const float ul = (float)(u - (double)uh);
-        const float4 v = make_float4((float)a, (float)W, uh, ul);
+        const float4 v = asm_axis_entry(A, (double)k * (double)k);
         out[c.first[k]] = v;
         if (c.second[k] >= 0) out[c.second[k]] = v;
     }

@@ -2,6 +2,8 @@
 // transfer-function factors).  Shared by the plan code and the host emulator.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
+
 #include <complex>
 #include <vector>
 
@@ -39,6 +41,24 @@ std::vector<float2> split_phase(int P);
 void fft64(std::vector<cd>& x);
 std::vector<cd> fresnel_axis_dft(int P, double pitch, double lambda, double z);
 cd fresnel_coeff(double dx, double dy, double lambda, double z, bool literal_scale);
+// One axis of the ASM phase split (cwo_h.cuh): the constants of a parameter set, and the table entry
+// {a, W, u_hi, u_lo} of the bins +-kt, kt^2 = k2 (the same FP64 operations on the host and the device;
+// x: with frac(K) and the sign of K folded in).
+struct AsmAxis {
+    double lam2, pd2;   // a = lambda^2 k2 / (P pitch)^2
+    double c1, c2;      // K a / 2 per kt^2, K a^2 / 8 per kt^4 (cycles)
+    double c0, su;      // W is reduced and less c0; u = su a
+};
+AsmAxis asm_axis(int P, double pitch, double lambda, double z, bool is_x);
+__host__ __device__ __forceinline__ float4 asm_axis_entry(const AsmAxis& A, double k2) {
+    const double a = A.lam2 * k2 / A.pd2;
+    const double p1 = A.c1 * k2, p2 = A.c2 * k2 * k2;
+    const double q = (p1 - floor(p1)) + (p2 - floor(p2));
+    const double W = (q - floor(q)) - A.c0;
+    const double u = A.su * a;
+    const float uh = (float)u;
+    return make_float4((float)a, (float)W, uh, (float)(u - (double)uh));
+}
 void asm_axis_table(const AxisGeo& g, double pitch, double lambda, double z, bool is_x, float4* out);
 // Shifted ASM (Eq. shift_ang2): the phase gains shift * f cycles (f = kt / (P pitch)), and bins
 // with |f - wc| > ww / 2 (ww > 0) are outside the Rect window: their entry gets a = 2, which the
