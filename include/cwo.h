@@ -270,6 +270,32 @@ cwo_status cwo_propagate_epilogue(cwo_plan* plan, const void* in_c64, void* out_
 cwo_status cwo_gs_run(cwo_plan* plan, const float* amplitude, void* field_c64, float* intensity, int batch,
                       int iterations, void* cuda_stream);
 
+/* The steps of a phase-only hologram optimisation around a propagation and its adjoint.  A phase
+ * [h][w] fills the window at column ox and row oy of an nx x ny canvas (any position and size inside
+ * it; nx even, nx, ny <= CWO_MAX_SIDE); every buffer is contiguous device memory of the current device
+ * owned by the caller, canvases complex64 [ny][nx], windows float [h][w]; canvases that are written
+ * start on a 16-byte boundary.  All are enqueued on cuda_stream.
+ *   field       field = exp(i phase) on the window, 0 elsewhere
+ *   intensity   |u|^2 on the window
+ *   loss        residual = |u|^2 - target on the window, loss = mean of its squares, summed in FP64 in a
+ *               fixed order; partial: CWO_HOLOGRAM_PARTIALS doubles of scratch
+ *   seed        2 u g s on the window, 0 elsewhere: with s = 1 (gloss NULL) the derivative by u
+ *               (conjugate Wirtinger, as torch.autograd) of a loss whose derivative by |u|^2 is g; with
+ *               gloss (one device float) s = 2 gloss / (h w), for g the residual above
+ *   phase_grad  Re(conj(g) i exp(i phase)) on the window: the derivative by the phase of a loss
+ *               whose derivative by the field is g */
+#define CWO_HOLOGRAM_PARTIALS 1216
+cwo_status cwo_hologram_field(const float* phase, int h, int w, int nx, int ny, int ox, int oy, void* field_c64,
+                              void* cuda_stream);
+cwo_status cwo_hologram_intensity(const void* u_c64, int h, int w, int nx, int ny, int ox, int oy, float* intensity,
+                                  void* cuda_stream);
+cwo_status cwo_hologram_loss(const void* u_c64, const float* target, int h, int w, int nx, int ny, int ox, int oy,
+                             float* residual, float* loss, double* partial, void* cuda_stream);
+cwo_status cwo_hologram_seed(const void* u_c64, const float* g, const float* gloss, int h, int w, int nx, int ny, int ox,
+                             int oy, void* out_c64, void* cuda_stream);
+cwo_status cwo_hologram_phase_grad(const void* g_c64, const float* phase, int h, int w, int nx, int ny, int ox, int oy,
+                                   float* gphase, void* cuda_stream);
+
 /* Number of kernel launches one call of cwo_propagate_batch makes for this plan (for launch
  * accounting in benchmarks): 3 for the angular spectrum types, 2 for the Fresnel Fourier form and
  * for the Fresnel convolution and shifted Fresnel types, whose separable line passes take 2 (3

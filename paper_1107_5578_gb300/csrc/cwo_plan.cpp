@@ -64,9 +64,9 @@ PFN_memGetAddressRange get_addr_range_fn() {
 }
 
 // Check that [ptr, ptr + bytes) is device memory of `device` inside one allocation.
-cwo_status check_device_range(const void* ptr, size_t bytes, int device, const char* name) {
+cwo_status check_device_range(const void* ptr, size_t bytes, int device, const char* name, int align = 8) {
     if (!ptr) return fail(CWO_ERR_INVALID_ARG, "%s is NULL", name);
-    if ((uintptr_t)ptr % 8 != 0) return fail(CWO_ERR_INVALID_ARG, "%s is not 8-byte aligned", name);
+    if ((uintptr_t)ptr % align != 0) return fail(CWO_ERR_INVALID_ARG, "%s is not %d-byte aligned", name, align);
     cudaPointerAttributes at;
     cudaError_t e = cudaPointerGetAttributes(&at, ptr);
     if (e != cudaSuccess) {
@@ -122,8 +122,8 @@ size_t tables_bytes(int nx, int ny) {
 
 void cwo::set_last_error(const char* msg) { g_err = msg ? msg : ""; }
 
-int cwo::check_device_buffer(const void* ptr, size_t bytes, int device, const char* name) {
-    return check_device_range(ptr, bytes, device, name);
+int cwo::check_device_buffer(const void* ptr, size_t bytes, int device, const char* name, int align) {
+    return check_device_range(ptr, bytes, device, name, align);
 }
 
 // ------------------------------------------------------------------------------------------

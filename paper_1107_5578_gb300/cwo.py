@@ -32,6 +32,7 @@ STATUS_NAMES = {0: "CWO_OK", 1: "CWO_ERR_INVALID_ARG", 2: "CWO_ERR_UNSUPPORTED",
                 4: "CWO_ERR_CUDA", 5: "CWO_ERR_TIMEOUT"}
 DEFAULT_WAVELENGTH = 633e-9
 DEFAULT_PITCH = 10e-6
+HOLOGRAM_PARTIALS = 1216
 
 _lock = threading.Lock()
 _lib = None
@@ -113,6 +114,11 @@ def lib() -> ctypes.CDLL:
                 "cwo_launches_per_call": ([vp], i),
                 "cwo_propagate_epilogue": ([vp, vp, vp, i, i, i, vp, vp, vp], i),
                 "cwo_gs_run": ([vp, vp, vp, vp, i, i, vp], i),
+                "cwo_hologram_field": ([vp, i, i, i, i, i, i, vp, vp], i),
+                "cwo_hologram_intensity": ([vp, i, i, i, i, i, i, vp, vp], i),
+                "cwo_hologram_loss": ([vp, vp, i, i, i, i, i, i, vp, vp, vp, vp], i),
+                "cwo_hologram_seed": ([vp, vp, vp, i, i, i, i, i, i, vp, vp], i),
+                "cwo_hologram_phase_grad": ([vp, vp, i, i, i, i, i, i, vp, vp], i),
                 "cwo_plan_check": ([vp], i),
                 "cwo_plan_set_timing_events": ([vp, ctypes.POINTER(ctypes.c_void_p)], i),
                 "cwo_last_error": ([], ctypes.c_char_p),

@@ -21,6 +21,97 @@ import torch
 from . import autograd, cwo, synth
 
 
+class _Geometry:
+    """The window of a problem on its canvas and the plan that propagates it, as they were at the call."""
+    __slots__ = ("plan", "args", "canvas")
+
+    def __init__(self, p: "HologramProblem"):
+        self.plan, self.canvas = p.plan, p.canvas
+        self.args = (p.h, p.w, p.canvas, p.canvas, p.ox, p.oy)
+
+    def propagated(self, phi):
+        """U = A exp(i phi) on the canvas"""
+        phi = phi.contiguous()
+        x = torch.empty(self.canvas, self.canvas, dtype=torch.complex64, device=phi.device)
+        _call("cwo_hologram_field", phi, *self.args, x)
+        return self.plan.propagate(x, out=x)
+
+    def phase_gradient(self, phi, u, gw, gl):
+        """A^H of the seed (through the adjoint kernels), and its derivative by the phase"""
+        phi, u, gw = phi.contiguous(), u.contiguous(), gw.contiguous()
+        g = torch.empty_like(u)
+        _call("cwo_hologram_seed", u, gw, gl, *self.args, g)
+        self.plan.adjoint(g, out=g)
+        out = torch.empty_like(phi)
+        _call("cwo_hologram_phase_grad", g, phi, *self.args, out)
+        return out
+
+    # the same steps as tensor operators: for inputs the kernels do not take, and for gradients of
+    # gradients
+    def field(self, phi):
+        h, w, _, _, ox, oy = self.args
+        x = torch.zeros(self.canvas, self.canvas, dtype=torch.complex64, device=phi.device)
+        x[oy:oy + h, ox:ox + w] = torch.polar(torch.ones_like(phi), phi)
+        return x
+
+    def intensity(self, phi):
+        h, w, _, _, ox, oy = self.args
+        u = autograd.propagate(self.field(phi), self.plan)
+        uw = u[oy:oy + h, ox:ox + w]
+        return uw.real ** 2 + uw.imag ** 2
+
+
+def _call(name, *args):
+    st = getattr(cwo.lib(), name)(*(a.data_ptr() if isinstance(a, torch.Tensor) else a for a in args), cwo._stream_handle(None))
+    if st != cwo.OK:
+        cwo.check(st, name)
+
+
+class _Intensity(torch.autograd.Function):
+    """phase [h][w] -> |A exp(i phase)|^2 on the window, through the fused kernels (cwo_holo.cu)."""
+
+    @staticmethod
+    def forward(ctx, phi, geo):
+        u = geo.propagated(phi)
+        out = torch.empty(phi.shape, dtype=torch.float32, device=phi.device)
+        _call("cwo_hologram_intensity", u, *geo.args, out)
+        ctx.geo = geo
+        ctx.save_for_backward(phi, u)
+        return out
+
+    @staticmethod
+    def backward(ctx, gi):
+        phi, u = ctx.saved_tensors
+        if torch.is_grad_enabled():   # a graph of the gradient is wanted: the composed operators have one
+            return torch.autograd.grad(ctx.geo.intensity(phi), phi, gi, create_graph=True)[0], None
+        return ctx.geo.phase_gradient(phi, u, gi.resolve_neg(), None), None
+
+
+class _Loss(torch.autograd.Function):
+    """phase [h][w], target -> mean squared difference between the intensity and the target.  The
+    residual is kept for the gradient, not the target, which the caller may change in the meantime."""
+
+    @staticmethod
+    def forward(ctx, phi, target, geo):
+        u = geo.propagated(phi)
+        residual = torch.empty(phi.shape, dtype=torch.float32, device=phi.device)
+        loss = torch.empty((), dtype=torch.float32, device=phi.device)
+        partial = torch.empty(cwo.HOLOGRAM_PARTIALS, dtype=torch.float64, device=phi.device)
+        _call("cwo_hologram_loss", u, target, *geo.args, residual, loss, partial)
+        ctx.geo = geo
+        ctx.save_for_backward(phi, u, residual)
+        return loss
+
+    @staticmethod
+    def backward(ctx, gl):
+        phi, u, residual = ctx.saved_tensors
+        if torch.is_grad_enabled():
+            inten = ctx.geo.intensity(phi)
+            d = inten - (inten.detach() - residual)
+            return torch.autograd.grad((d * d).mean(), phi, gl, create_graph=True)[0], None, None
+        return ctx.geo.phase_gradient(phi, u, residual, gl.resolve_neg()), None, None
+
+
 class HologramProblem:
     def __init__(self, h=1080, w=1920, canvas=2048, pitch=6.4e-6, wavelength=520e-9, z=0.15,
                  seed=1, device="cuda"):
@@ -39,17 +130,26 @@ class HologramProblem:
         self.target = torch.from_numpy(self.target_np).float().to(self.device)
 
     def field(self, phi: torch.Tensor) -> torch.Tensor:
-        x = torch.zeros(self.canvas, self.canvas, dtype=torch.complex64, device=phi.device)
-        x[self.oy:self.oy + self.h, self.ox:self.ox + self.w] = torch.polar(torch.ones_like(phi), phi)
-        return x
+        return _Geometry(self).field(phi)
+
+    def _window(self, t) -> bool:
+        """t is what the fused kernels take: a plain float32 CUDA tensor [h][w]"""
+        return type(t) in (torch.Tensor, torch.nn.Parameter) and t.dtype == torch.float32 and t.is_cuda \
+            and t.shape == (self.h, self.w) and not t.is_neg()
+
+    def _fused(self, phi) -> bool:
+        return self._window(phi) and self.plan.nx == self.plan.ny == self.canvas \
+            and 0 <= self.oy <= self.canvas - self.h and 0 <= self.ox <= self.canvas - self.w
 
     def intensity(self, phi: torch.Tensor) -> torch.Tensor:
-        u = autograd.propagate(self.field(phi), self.plan)
-        uw = u[self.oy:self.oy + self.h, self.ox:self.ox + self.w]
-        return uw.real ** 2 + uw.imag ** 2
+        geo = _Geometry(self)
+        return _Intensity.apply(phi, geo) if self._fused(phi) else geo.intensity(phi)
 
     def loss(self, phi: torch.Tensor) -> torch.Tensor:
-        d = self.intensity(phi) - self.target
+        geo, t = _Geometry(self), self.target
+        if self._fused(phi) and self._window(t) and t.is_contiguous() and not t.requires_grad and t.device == phi.device:
+            return _Loss.apply(phi, t, geo)
+        d = self.intensity(phi) - t
         return (d * d).mean()
 
 
