@@ -18,14 +18,16 @@ extern "C" {
 /* Axis index -> frequency bin (0 .. p-1) for a padded axis of length p (power of two in
  * [32, 8192]).  Index idx = e*(p/16) + t is register e of thread t in the last forward FFT stage,
  * which holds the output at digit-reversed (DIF) position 16 t + e; along x the same index is
- * the storage column of the 2Nx-wide intermediate.  bins: p ints, caller-owned. */
+ * the storage column of the 2Nx-wide intermediate (below p = 8192, where that is the split index of
+ * cwo_debug_split_axis).  bins: p ints, caller-owned. */
 cwo_status cwo_debug_axis_bins(int p, int* bins);
 
 /* Split order of a zero-padded axis of length p (power of two in [64, 8192]): the p-point DFT of
  * p/2 samples x_n is, exactly, the (p/2)-point DFT of x_n at the even frequencies and that of
  * x_n W_p^n at the odd ones.  Split index i = h (p/2) + idx (h = 0: even, 1: odd; idx a
- * (p/2)-point axis index, see cwo_debug_axis_bins) holds frequency 2 bin(idx) + h.  The column
- * pass at p = 8192 with a cached transfer function stores that table's rows in this order.
+ * (p/2)-point axis index, see cwo_debug_axis_bins) holds frequency 2 bin(idx) + h.  At p = 8192 the
+ * row passes leave the intermediate's columns in this order, and the column pass with a cached
+ * transfer function stores that table's rows in it.
  * index: p ints, the p-point axis index of the same frequency; phase_ri: p floats, W_p^n =
  * exp(-2 pi i n / p) for n < p/2 (re, im interleaved) rounded from FP64.  Caller-owned; either
  * may be NULL. */

@@ -151,7 +151,7 @@ extern "C" cwo_status cwo_debug_emulate(int nx, int ny, double dx, double dy, do
         return CWO_ERR_INVALID_ARG;
     const int px = 2 * nx, py = 2 * ny;
     const AxisGeo gx(px), gy(py);
-    const std::vector<float4> twx = twiddle_table(gx), twy = twiddle_table(gy);
+    const std::vector<float4>&twx = twiddle_table(gx), &twy = twiddle_table(gy);
     std::vector<float4> ax(px), ay(py);
     std::vector<float2> hx(px), hy(py);
     float K = 0.f;
@@ -196,9 +196,9 @@ extern "C" cwo_status cwo_debug_emulate(int nx, int ny, double dx, double dy, do
         // cache builder does (split index i at the y axis index of its frequency) for the
         // canonical column of the mirror pair
         constexpr int Q = kSplitColP / 2;
-        const std::vector<float4> twq = twiddle_table(AxisGeo(Q));
-        const std::vector<float2> wn = split_phase(py);
-        const std::vector<int> yi = split_axis_index(py);
+        const std::vector<float4>& twq = twiddle_table(AxisGeo(Q));
+        const std::vector<float2>& wn = split_phase(py);
+        const std::vector<int>& yi = split_axis_index(py);
         const std::vector<int2> prs = mirror_pairs(gx);
         std::vector<float2> hs(py);
         for (const int2& pr : prs) {
@@ -238,7 +238,7 @@ extern "C" cwo_status cwo_debug_emulate_shifted(int nx, int ny, double dx, doubl
     const int px = 2 * nx, py = 2 * ny;
     const int tmode = asm_tail_mode(px, py, dx, dy, lambda, z);
     if (tmode == 2) return CWO_ERR_UNSUPPORTED;   // the per-element FP64 arm is not emulated here
-    const std::vector<float4> twx = twiddle_table(AxisGeo(px)), twy = twiddle_table(AxisGeo(py));
+    const std::vector<float4>&twx = twiddle_table(AxisGeo(px)), &twy = twiddle_table(AxisGeo(py));
     std::vector<float4> ax(px), ay(py);
     asm_axis_table_shifted(AxisGeo(px), dx, lambda, z, true, sh->ox, sh->cx, sh->wx, ax.data());
     asm_axis_table_shifted(AxisGeo(py), dy, lambda, z, false, sh->oy, sh->cy, sh->wy, ay.data());
@@ -275,7 +275,7 @@ extern "C" cwo_status cwo_debug_emulate_shifted_fresnel(int nx, int ny, double d
         !std::isfinite(z) || z == 0.0)
         return CWO_ERR_INVALID_ARG;
     const int px = 2 * nx, py = 2 * ny;
-    const std::vector<float4> twx = twiddle_table(AxisGeo(px)), twy = twiddle_table(AxisGeo(py));
+    const std::vector<float4>&twx = twiddle_table(AxisGeo(px)), &twy = twiddle_table(AxisGeo(py));
     std::vector<float2> fx(nx), fy(ny), qx(nx), qy(ny), hx(px), hy(py);
     const double cph = 6.283185307179586476925286766559 * frac01(z / lambda);
     const cd C = cd(std::cos(cph), std::sin(cph)) / cd(0.0, lambda * z) * (dx0 * dy0);
@@ -338,7 +338,7 @@ extern "C" cwo_status cwo_debug_line_fft(int p, int inverse, const float* in_ri,
     using namespace cwo::host;
     if (!in_ri || !out_ri || p < 32 || p > 8192 || (p & (p - 1))) return CWO_ERR_INVALID_ARG;
     const AxisGeo g(p);
-    const std::vector<float4> tw = twiddle_table(g);
+    const std::vector<float4>& tw = twiddle_table(g);
     if (!inverse) pick_fwd(p)((const float2*)in_ri, 1, (float2*)out_ri, 1, tw.data());
     else pick_inv(p)((const float2*)in_ri, 1, (float2*)out_ri, 1, tw.data());
     return CWO_OK;

@@ -46,7 +46,8 @@ cudaError_t launch_asm_tables(const AsmItemList& list, int items, const int* kbx
 
 // Transfer-function description for the column pass.  Per-axis tables are indexed by the axis
 // index idx = e * T + t (register e of thread t in the last forward stage, i.e. DIF position
-// 16 t + e); along x the same index is the storage column of the intermediate.
+// 16 t + e), in split order along x at Px = 8192; along x the index is the storage column of the
+// intermediate.
 struct HParams {
     int mode;                 // HMode
     int conj;                 // 1: adjoint (conj H)
@@ -138,7 +139,9 @@ cudaError_t launch_col_stack(int py, const float2* win, float2* wout, long long 
 // entry i is evaluated at y axis index yidx[i] (the split order of k_col_split).
 cudaError_t launch_build_hcache(float2* out, int npairs, int py, const HParams& hp, cudaStream_t st,
                                 const int* yidx = nullptr);
-// Py of the split column pass (a transfer function cached per plan)
+// Padded axis of the split forms: the row passes along x, and along y the column pass with a transfer
+// function cached per plan.  Their twiddles (tw of the row launchers at this Px, hp.split_tw) are those
+// of the half-length transform followed by W_P^n
 constexpr int kSplitColP = 8192;
 // Fresnel diffraction in Fourier form (cwo_fourier.cu): source chirp + row FFT into the
 // [items][Px = Nx][Ny] intermediate; column FFT + destination chirp into the centred output

@@ -115,6 +115,10 @@ size_t tables_bytes(int nx, int ny) {
     b += (size_t)(gx.tw_off(gx.NST - 1) + gy.tw_off(gy.NST - 1)) * sizeof(float4);
     b += (size_t)(gx.P + gy.P) * sizeof(int);
     b += (size_t)(gx.P + gy.P) * sizeof(float4) + sizeof(float) * 2;
+    if (gx.P == cwo::kSplitColP || gy.P == cwo::kSplitColP) {   // split constants, the x table of the line pass
+        const AxisGeo gq(cwo::kSplitColP / 2);
+        b += (size_t)gq.tw_off(gq.NST - 1) * sizeof(float4) + (size_t)(gq.P + gx.P) * sizeof(float2);
+    }
     return b;
 }
 
@@ -156,8 +160,8 @@ struct cwo_plan {
     cwo_type type = CWO_ANGULAR;
     unsigned flags = 0;
     int device = 0;
-    float4* tw_x = nullptr;   // twiddles along x (rows, length px)
-    float4* tw_y = nullptr;   // twiddles along y (columns, length py); aliases tw_x if px == py
+    float4* tw_x = nullptr;   // twiddles along x (rows, length px); split_tw at px = 8192
+    float4* tw_y = nullptr;   // twiddles along y (columns, length py); aliases tw_x if px == py < 8192
     int* kb_x = nullptr;
     int* kb_y = nullptr;
     int2* pairs_x = nullptr;   // mirror storage-column pairs along x
@@ -200,16 +204,26 @@ struct cwo_plan {
     cwo_shifted_fresnel sfr{};
     // CWO_FLAG_CACHE_H: the ASM transfer function of the plan's own z, [Px/2 + 1 pairs][Py]
     float2* hcache = nullptr;
-    // with it at Py = 8192 (split column pass): the 4096-point twiddles, then W_8192^n (float2)
+    // an axis of 8192 points in the split form (the row passes, and the column pass with a cached
+    // transfer function): the 4096-point twiddles, then W_8192^n (float2).  Every table along x is then
+    // in the split order, but for the Fresnel line pass: its 8192-point twiddles tw_lx (tw_x below
+    // 8192) and its x tables hxl / zhxl in DIF order (xsplit_idx: the DIF index of each split index)
     float4* split_tw = nullptr;
     float2* split_w = nullptr;
+    float4* tw_lx = nullptr;
+    float2* hxl = nullptr;
+    float2* zhxl = nullptr;
+    const std::vector<int>* xsplit_idx = nullptr;
+    bool xsplit() const { return px == cwo::kSplitColP; }
+    AxisGeo gx() const { return AxisGeo(px, xsplit()); }
 };
 
 namespace {
 
 void free_plan(cwo_plan* p) {
     if (!p) return;
-    cudaFree(p->tw_x);
+    if (p->tw_lx != p->tw_x && p->tw_lx != p->tw_y) cudaFree(p->tw_lx);
+    if (p->tw_x != p->split_tw) cudaFree(p->tw_x);
     if (p->tw_y != p->tw_x) cudaFree(p->tw_y);
     cudaFree(p->kb_x); cudaFree(p->kb_y); cudaFree(p->pairs_x);
     cudaFree(p->ax); cudaFree(p->ay); cudaFree(p->hx); cudaFree(p->hy); cudaFree(p->kf);
@@ -224,6 +238,7 @@ void free_plan(cwo_plan* p) {
     cudaFree(p->fpre_cx); cudaFree(p->fpre_cy); cudaFree(p->fpost_cx); cudaFree(p->fpost_cy);
     cudaFree(p->hcache);
     cudaFree(p->split_tw);
+    cudaFree(p->hxl); cudaFree(p->zhxl);
     delete p;
 }
 
@@ -258,13 +273,27 @@ cwo_status check_params(int nx, int ny, double dx, double dy, double lambda, dou
 // host tables of one parameter set
 void host_h_tables(const cwo_plan* p, double z, float4* ax, float4* ay, float2* hx, float2* hy, float* kf) {
     if (p->shifted) {
-        asm_axis_table_shifted(AxisGeo(p->px), p->dx, p->lambda, z, true, p->shift.ox, p->shift.cx, p->shift.wx, ax);
+        asm_axis_table_shifted(p->gx(), p->dx, p->lambda, z, true, p->shift.ox, p->shift.cx, p->shift.wx, ax);
         asm_axis_table_shifted(AxisGeo(p->py), p->dy, p->lambda, z, false, p->shift.oy, p->shift.cy, p->shift.wy, ay);
         if (kf) *kf = (float)(z / p->lambda);
         return;
     }
     make_h_tables(p->px, p->py, p->dx, p->dy, p->lambda, z, p->type == CWO_FRESNEL_CONV,
-                  (p->flags & CWO_FLAG_LITERAL_SCALE) != 0, ax, ay, hx, hy, kf);
+                  (p->flags & CWO_FLAG_LITERAL_SCALE) != 0, ax, ay, hx, hy, kf, p->xsplit());
+}
+
+// a Fresnel x table in the DIF order of the line pass
+void line_order(const cwo_plan* p, const float2* hx, float2* hxl) {
+    for (int i = 0; i < p->px; ++i) hxl[(*p->xsplit_idx)[i]] = hx[i];
+}
+
+// the plan's own, where it has one
+cwo_status line_table(cwo_plan* p, const std::vector<float2>& hx) {
+    if (!p->xsplit_idx) return CWO_OK;
+    std::vector<float2> hxl(p->px);
+    line_order(p, hx.data(), hxl.data());
+    const cwo_status st = dev_alloc(&p->hxl, hxl.size(), "x table");
+    return st ? st : upload(p->hxl, hxl, "x table upload");
 }
 
 cwo_status ensure_scratch(cwo_plan* p, int items) {
@@ -331,8 +360,8 @@ cwo_status ensure_ztables(cwo_plan* p, int items) {
     p->zs_cached.clear();
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize before growing tables");
-    cudaFree(p->zax); cudaFree(p->zay); cudaFree(p->zhx); cudaFree(p->zhy); cudaFree(p->zkf);
-    p->zax = p->zay = nullptr; p->zhx = p->zhy = nullptr; p->zkf = nullptr;
+    cudaFree(p->zax); cudaFree(p->zay); cudaFree(p->zhx); cudaFree(p->zhy); cudaFree(p->zkf); cudaFree(p->zhxl);
+    p->zax = p->zay = nullptr; p->zhx = p->zhy = p->zhxl = nullptr; p->zkf = nullptr;
     p->zstage.release();
     p->zcap = 0;
     cwo_status st;
@@ -343,9 +372,11 @@ cwo_status ensure_ztables(cwo_plan* p, int items) {
             (st = dev_alloc(&p->zkf, (size_t)items, "per-item K")))
             return st;   // filled on the device: no staging
     } else {
-        if ((st = dev_alloc(&p->zhx, nx4, "per-item x tables")) || (st = dev_alloc(&p->zhy, ny4, "per-item y tables")))
+        const size_t nxl = p->xsplit_idx ? nx4 : 0;
+        if ((st = dev_alloc(&p->zhx, nx4, "per-item x tables")) || (st = dev_alloc(&p->zhy, ny4, "per-item y tables")) ||
+            (st = dev_alloc(&p->zhxl, nxl, "per-item x tables")))
             return st;
-        zbytes = (nx4 + ny4) * sizeof(float2);
+        zbytes = (nx4 + ny4 + nxl) * sizeof(float2);
     }
     if (zbytes && (st = staging_alloc(p->zstage, zbytes))) return st;
     p->zcap = items;
@@ -521,9 +552,14 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
             if ((st = staging_acquire(p->zstage, &hb, &zslot))) return st;
             float2* hhx = (float2*)hb;
             float2* hhy = hhx + (size_t)batch * p->px;
-            for (int i = 0; i < batch; ++i)
+            float2* hhxl = hhy + (size_t)batch * p->py;
+            for (int i = 0; i < batch; ++i) {
                 host_h_tables(p, zs[i], nullptr, nullptr, hhx + (size_t)i * p->px, hhy + (size_t)i * p->py, nullptr);
+                if (p->zhxl) line_order(p, hhx + (size_t)i * p->px, hhxl + (size_t)i * p->px);
+            }
             cudaError_t e;
+            if (p->zhxl && (e = cudaMemcpyAsync(p->zhxl, hhxl, (size_t)batch * p->px * sizeof(float2), cudaMemcpyHostToDevice, s)))
+                return cuda_fail(e, "table upload");
             if ((e = cudaMemcpyAsync(p->zhx, hhx, (size_t)batch * p->px * sizeof(float2), cudaMemcpyHostToDevice, s)) ||
                 (e = cudaMemcpyAsync(p->zhy, hhy, (size_t)batch * p->py * sizeof(float2), cudaMemcpyHostToDevice, s)))
                 return cuda_fail(e, "table upload");
@@ -544,6 +580,7 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
         }
     }
 
+    const float2* line_hx = !p->xsplit_idx ? hp.hx : zs ? p->zhxl : p->hxl;
     const long long wstride = (long long)p->ny * p->px;
     const bool timing = p->tev[0] != nullptr;
     auto mark = [&](int i) { return timing ? cudaEventRecord(p->tev[i], s) : cudaSuccess; };
@@ -593,8 +630,8 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
             return cuda_fail(e, "tensor map of the output");
         const long long istr = in_stride ? in_stride : field;
         if ((e = mark(0)) ||
-            (e = cwo::launch_line_conv(p->px, fin, istr, &p->wmap_s, p->ny, batch, hp.hx, hp.x_item_stride, hp.conj,
-                                       (float)(1.0 / p->px), p->tw_x, p->status, prex, postx, s)) ||
+            (e = cwo::launch_line_conv(p->px, fin, istr, &p->wmap_s, p->ny, batch, line_hx, hp.x_item_stride, hp.conj,
+                                       (float)(1.0 / p->px), p->tw_lx, p->status, prex, postx, s)) ||
             (e = mark(1)) ||
             (e = cwo::launch_line_conv(p->py, p->scratch, field, &omap, p->nx, batch, hp.hy, hp.y_item_stride, hp.conj,
                                        (float)(1.0 / p->py), p->tw_y, p->status, prey, posty, s)) ||
@@ -667,7 +704,7 @@ cwo_status ensure_itables(cwo_plan* p, int items) {
 void fresnel_item_tables(const cwo_plan* p, const cwo_item& it, float4* xt, float4* yt, bool lines) {
     std::vector<float2> hx(p->px), hy(p->py);
     make_h_tables(p->px, p->py, it.dx, it.dy, it.lambda, it.z, true, (it.flags & CWO_FLAG_LITERAL_SCALE) != 0,
-                  nullptr, nullptr, hx.data(), hy.data(), nullptr);
+                  nullptr, nullptr, hx.data(), hy.data(), nullptr, p->xsplit() && !lines);
     if (lines) {
         std::copy(hx.begin(), hx.end(), (float2*)xt);
         std::copy(hy.begin(), hy.end(), (float2*)yt);
@@ -780,7 +817,7 @@ cwo_status run_items(cwo_plan* p, const void* in, long long in_stride, void* out
                 return cuda_fail(e, "tensor map of the output");
             if ((e = cwo::launch_line_conv(p->px, fin + i0 * in_stride, in_stride, &p->wmap_s, p->ny, n,
                                            (const float2*)(p->ix + (size_t)i0 * p->px), 2LL * p->px, 0,
-                                           (float)(1.0 / p->px), p->tw_x, p->status, nullptr, nullptr, s)) ||
+                                           (float)(1.0 / p->px), p->tw_lx, p->status, nullptr, nullptr, s)) ||
                 (last && (e = mark(1))) ||
                 (e = cwo::launch_line_conv(p->py, p->scratch, field, &omap, p->nx, n,
                                            (const float2*)(p->iy + (size_t)i0 * p->py), 2LL * p->py, 0,
@@ -872,15 +909,39 @@ cwo_status create_impl(int nx, int ny, double dx, double dy, double lambda, doub
     cudaError_t e = cudaGetDevice(&p->device);
     if (e != cudaSuccess) { free_plan(p); return cuda_fail(e, "cudaGetDevice"); }
 
-    const AxisGeo gx(p->px), gy(p->py);
-    const std::vector<float4> twx = twiddle_table(gx);
+    const AxisGeo gx = p->gx(), gy(p->py);
     const std::vector<int> kbx = bin_table(gx), kby = bin_table(gy);
-    if ((st = dev_alloc(&p->tw_x, twx.size(), "x twiddles")) || (st = upload(p->tw_x, twx, "x twiddle upload"))) { free_plan(p); return st; }
-    if (p->py == p->px) {
+    if (p->px == cwo::kSplitColP || p->py == cwo::kSplitColP) {
+        const std::vector<float4>& twq = twiddle_table(AxisGeo(cwo::kSplitColP / 2));
+        const std::vector<float2>& wn = split_phase(cwo::kSplitColP);
+        const size_t n4 = twq.size() + (wn.size() + 1) / 2;
+        if ((st = dev_alloc(&p->split_tw, n4, "split twiddles")) || (st = upload(p->split_tw, twq, "split twiddle upload"))) {
+            free_plan(p);
+            return st;
+        }
+        p->split_w = reinterpret_cast<float2*>(p->split_tw + twq.size());
+        if ((st = upload(p->split_w, wn, "split phase upload"))) { free_plan(p); return st; }
+    }
+    if (p->xsplit()) {
+        p->tw_x = p->split_tw;
+    } else {
+        const std::vector<float4>& twx = twiddle_table(gx);
+        if ((st = dev_alloc(&p->tw_x, twx.size(), "x twiddles")) || (st = upload(p->tw_x, twx, "x twiddle upload"))) { free_plan(p); return st; }
+    }
+    if (p->py == p->px && !p->xsplit()) {
         p->tw_y = p->tw_x;
     } else {
-        const std::vector<float4> twy = twiddle_table(gy);
+        const std::vector<float4>& twy = twiddle_table(gy);
         if ((st = dev_alloc(&p->tw_y, twy.size(), "y twiddles")) || (st = upload(p->tw_y, twy, "y twiddle upload"))) { free_plan(p); return st; }
+    }
+    p->tw_lx = p->tw_x;
+    if (p->xsplit()) {
+        p->tw_lx = p->tw_y;
+        if (p->py != p->px) {
+            const std::vector<float4>& twx = twiddle_table(AxisGeo(p->px));
+            if ((st = dev_alloc(&p->tw_lx, twx.size(), "x twiddles")) || (st = upload(p->tw_lx, twx, "x twiddle upload"))) { free_plan(p); return st; }
+        }
+        if (type == CWO_FRESNEL_CONV || type == CWO_SHIFTED_FRESNEL) p->xsplit_idx = &split_axis_index(p->px);
     }
     const std::vector<int2> prs = mirror_pairs(gx);
     if ((st = dev_alloc(&p->pairs_x, prs.size(), "x pairs")) || (st = upload(p->pairs_x, prs, "x pair upload"))) { free_plan(p); return st; }
@@ -891,7 +952,7 @@ cwo_status create_impl(int nx, int ny, double dx, double dy, double lambda, doub
         const double cph = 2.0 * kPi * frac01(z / lambda);
         cd C = cd(std::cos(cph), std::sin(cph)) / cd(0.0, lambda * z);
         if (!(flags & CWO_FLAG_LITERAL_SCALE)) C *= dx * dy;
-        shifted_fresnel_axis(nx, dx, p->sfr.dx1, p->sfr.ox0, p->sfr.ox1, lambda, z, C, fx.data(), qx.data(), hx.data());
+        shifted_fresnel_axis(nx, dx, p->sfr.dx1, p->sfr.ox0, p->sfr.ox1, lambda, z, C, fx.data(), qx.data(), hx.data(), p->xsplit());
         shifted_fresnel_axis(ny, dy, p->sfr.dy1, p->sfr.oy0, p->sfr.oy1, lambda, z, cd(1.0, 0.0), fy.data(), qy.data(), hy.data());
         auto conj = [](std::vector<float2> v) { for (auto& a : v) a.y = -a.y; return v; };
         const std::vector<float2> cqx = conj(qx), cqy = conj(qy), cfx = conj(fx), cfy = conj(fy);
@@ -904,7 +965,8 @@ cwo_status create_impl(int nx, int ny, double dx, double dy, double lambda, doub
             (st = dev_alloc(&p->fpost_cx, nx, "x adjoint factor")) || (st = upload(p->fpost_cx, cfx, "upload")) ||
             (st = dev_alloc(&p->fpost_cy, ny, "y adjoint factor")) || (st = upload(p->fpost_cy, cfy, "upload")) ||
             (st = dev_alloc(&p->hx, hx.size(), "x table")) || (st = upload(p->hx, hx, "x table upload")) ||
-            (st = dev_alloc(&p->hy, hy.size(), "y table")) || (st = upload(p->hy, hy, "y table upload"))) {
+            (st = dev_alloc(&p->hy, hy.size(), "y table")) || (st = upload(p->hy, hy, "y table upload")) ||
+            (st = line_table(p, hx))) {
             free_plan(p);
             return st;
         }
@@ -933,7 +995,8 @@ cwo_status create_impl(int nx, int ny, double dx, double dy, double lambda, doub
         std::vector<float2> hx(p->px), hy(p->py);
         host_h_tables(p, z, nullptr, nullptr, hx.data(), hy.data(), nullptr);
         if ((st = dev_alloc(&p->hx, hx.size(), "x table")) || (st = upload(p->hx, hx, "x table upload")) ||
-            (st = dev_alloc(&p->hy, hy.size(), "y table")) || (st = upload(p->hy, hy, "y table upload"))) { free_plan(p); return st; }
+            (st = dev_alloc(&p->hy, hy.size(), "y table")) || (st = upload(p->hy, hy, "y table upload")) ||
+            (st = line_table(p, hx))) { free_plan(p); return st; }
     }
     if ((st = dev_alloc(&p->status, 1, "status word"))) { free_plan(p); return st; }
     if ((e = cudaMemset(p->status, 0, sizeof(int))) != cudaSuccess) { free_plan(p); return cuda_fail(e, "cudaMemset"); }
@@ -943,17 +1006,8 @@ cwo_status create_impl(int nx, int ny, double dx, double dy, double lambda, doub
         if ((st = dev_alloc(&p->hcache, (size_t)npairs * p->py, "transfer-function cache"))) { free_plan(p); return st; }
         int* yidx = nullptr;   // the split order of the split column pass
         if (p->py == cwo::kSplitColP) {
-            const std::vector<float4> twq = twiddle_table(AxisGeo(p->py / 2));
-            const std::vector<float2> wn = split_phase(p->py);
-            const std::vector<int> yi = split_axis_index(p->py);
-            const size_t n4 = twq.size() + (wn.size() + 1) / 2;
-            if ((st = dev_alloc(&p->split_tw, n4, "split twiddles")) || (st = upload(p->split_tw, twq, "split twiddle upload"))) {
-                free_plan(p);
-                return st;
-            }
-            p->split_w = reinterpret_cast<float2*>(p->split_tw + twq.size());
-            if ((st = upload(p->split_w, wn, "split phase upload")) || (st = dev_alloc(&yidx, yi.size(), "split index")) ||
-                (st = upload(yidx, yi, "split index upload"))) {
+            const std::vector<int>& yi = split_axis_index(p->py);
+            if ((st = dev_alloc(&yidx, yi.size(), "split index")) || (st = upload(yidx, yi, "split index upload"))) {
                 cudaFree(yidx);
                 free_plan(p);
                 return st;
@@ -1174,11 +1228,11 @@ cwo_status cwo_debug_axis_bins(int p, int* bins) {
 cwo_status cwo_debug_split_axis(int p, int* index, float* phase_ri) {
     if (p < 64 || p > 8192 || (p & (p - 1))) return fail(CWO_ERR_INVALID_ARG, "bad axis length");
     if (index) {
-        const std::vector<int> v = split_axis_index(p);
+        const std::vector<int>& v = split_axis_index(p);
         std::copy(v.begin(), v.end(), index);
     }
     if (phase_ri) {
-        const std::vector<float2> w = split_phase(p);
+        const std::vector<float2>& w = split_phase(p);
         for (size_t n = 0; n < w.size(); ++n) { phase_ri[2 * n] = w[n].x; phase_ri[2 * n + 1] = w[n].y; }
     }
     return CWO_OK;
@@ -1195,7 +1249,7 @@ cwo_status cwo_debug_fresnel_axis(int p, double pitch, double lambda, double z, 
 cwo_status cwo_debug_twiddles(int p, float* out_ri) {
     if (!out_ri || p < 32 || p > 8192 || (p & (p - 1))) return fail(CWO_ERR_INVALID_ARG, "bad axis length");
     const AxisGeo g(p);
-    const std::vector<float4> tw = twiddle_table(g);
+    const std::vector<float4>& tw = twiddle_table(g);
     for (size_t i = 0; i < tw.size(); ++i) {
         out_ri[4 * i] = tw[i].x; out_ri[4 * i + 1] = tw[i].y; out_ri[4 * i + 2] = tw[i].z; out_ri[4 * i + 3] = tw[i].w;
     }

@@ -13,7 +13,7 @@
 // The intermediate W is COLUMN-MAJOR, [items][Px][Ny] complex64: storage column st holds the Ny
 // values of one frequency kx contiguously, so that the column pass streams whole columns.  Along
 // x the storage order is the register order of the last forward stage: register e of thread t
-// (DIF position 16 t + e) is storage column e * T + t.  A CTA handles R rows and transposes them
+// (DIF position 16 t + e) is storage column e * T + t (at Px = 8192 the split order below).  A CTA handles R rows and transposes them
 // through a dense shared-memory tile [st][r]; the tile moves to and from the intermediate as TMA
 // tensor boxes of R rows x 256 columns (R * 8 contiguous bytes per column), so the transposed
 // global side costs the threads no load/store instructions.
@@ -36,10 +36,6 @@ namespace cwo {
 // of each sector served from L2 to the neighbouring CTA) allow more CTAs per SM.  A TMA box must
 // span at least 16 contiguous bytes, hence >= 2 rows.
 template <int P> constexpr int rows_fwd() { return P >= 256 ? 4 : 8; }
-// at P = 8192 a CTA holds 2 rows (a pair per thread, 512 threads, 139 KB of exchange space): a
-// cluster of two CTAs forms each 4-row group, so that every stored column piece is a whole
-// 32-byte sector
-template <int P> constexpr bool rows_fwd_cluster() { return P >= 8192; }
 template <int P> constexpr int rows_inv() { return P >= 4096 ? 2 : (P >= 256 ? 4 : 8); }
 constexpr bool kRowInvPersistent = true;   // measured: 25.4 -> 23.0 us per 2048^2 field
 
@@ -205,113 +201,158 @@ k_row_fwd_p(const float2* __restrict__ in, long long in_item_stride, const __gri
     if (threadIdx.x == 0) tma_store_wait_read();
 }
 
-// Forward, cluster pair (P = 8192): CTA rank q of a two-CTA cluster transforms rows y0 + 2q and
-// y0 + 2q + 1 of a 4-row group, one thread per pair of rows (the two rows share every twiddle
-// load and move with 128-bit exchanges).  After both CTAs have finished their FFT exchanges
-// (cluster barrier), every thread writes both rows' values of each of its storage columns with one
-// 16-byte store into the 4-row tile of the CTA that stores that column half -- its own half
-// locally, the other half into the partner's shared memory -- and after a second cluster barrier
-// each CTA stores its [P/2 columns][4 rows] tile by TMA: 32 contiguous bytes per column.  Both
-// CTAs execute the same sequence of cluster barriers on every path (a bounded wait that expires
-// leaves the status bit set and the loop running), so neither can wait for a partner that has
-// left.  BULK: the rows are staged by bulk copies (16-byte aligned input); otherwise each thread
-// loads its own samples.  Measured against one row per thread (1024 threads, 8-byte tile stores):
-// 156.5 against 168.3 us per 4096^2 field.
+// ------------------------------------------------------------------------------------------
+// Split row passes (P = 8192 = 2 Q).  A row holds Q samples zero-padded to 2 Q, so its transform is
+// exactly the Q-point transforms of x_n (the even frequencies) and of x_n W_P^n (the odd ones), and
+// the cropped inverse is the Q-point inverse of the even half plus W_P^-n times that of the odd half.
+// The storage order along x is the split one: column h Q + e T + t holds frequency 2 k + h, k the
+// Q-point frequency of register e of thread t.  Against the 8192-point transform (radix 16, 16, 16,
+// 2) a row takes two exchanges of Q points per half instead of three of 2 Q, the tables of the
+// Q-point transform (34 against 70 KB), and each half is a tile of its own, so that one half's copy
+// runs beside the other's transform.  tw points to the Q-point twiddles, followed by W_P^n for n < Q.
+// Measured, two 4096^2 fields: forward 244 us against 313 for a pair of CTAs sharing four-row tiles
+// through distributed shared memory, inverse 238 against 318 for one tile buffer per CTA; the copies
+// alone (no transforms) took 254 and 228 in those forms, so both now run at the rate at which TMA
+// moves 32- and 16-byte column pieces.
+// ------------------------------------------------------------------------------------------
 template <int P>
-__host__ __device__ constexpr size_t row_fwd_c_xwords() { return 2 * (size_t)PairLayout<P, 1>::SLOTS; }
-template <int P>
-__host__ __device__ constexpr size_t row_fwd_c_smem_bytes() {
-    return (row_fwd_c_xwords<P>() + 2 * (size_t)stage_stride<P, 2>()) * sizeof(float2) + sizeof(uint64_t);
+__device__ __forceinline__ const float2* split_phase_of(const float4* tw) {
+    return reinterpret_cast<const float2*>(tw + Geo<P / 2>::TW_WORDS);
 }
 
-template <int P, bool PRE, bool BULK>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P / 16, 1)
-k_row_fwd_c(const float2* __restrict__ in, long long in_item_stride, const __grid_constant__ CUtensorMap wmap,
-             int item_off, int groups_per_item, int total_groups, const float4* __restrict__ tw, int* status,
-             const Prefactor pre) {
+// Forward: a CTA of 1024 threads walks groups of R = 4 rows, half by half (whole 32-byte sectors of
+// each stored column, without a partner CTA).  The samples of the next half are loaded into registers
+// as soon as the current tile is written, so that the loads overlap its TMA store; the store drains
+// behind the first stage.  The second half reads the same rows again, from L2.
+template <int P, int R, bool PRE>
+__global__ void __launch_bounds__(R * (P / 32), 1)
+k_row_fwd_s(const float2* __restrict__ in, long long in_item_stride, const __grid_constant__ CUtensorMap wmap,
+            int item_off, int groups_per_item, int total_groups, const float4* __restrict__ tw, const Prefactor pre) {
     pdl_wait();
-    constexpr int T = P / 16, N = P / 2, SST = stage_stride<P, 2>(), HALF = P / 2;
-    constexpr int BOX = kTmaBoxCols;
-    constexpr size_t XW = row_fwd_c_xwords<P>();
-    static_assert(XW >= (size_t)4 * HALF, "the 4-row half tile fits the exchange region");
+    constexpr int Q = P / 2, T = Q / 16, NT = R * T, BOX = kTmaBoxCols;
     extern __shared__ __align__(1024) float2 sm[];
-    float4* sx = reinterpret_cast<float4*>(sm);
-    float2* stage = sm + XW;
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(stage + 2 * SST);
-    const unsigned rank = cluster_ctarank();
-    const unsigned tile_remote = cluster_map(smem_u32(sm), rank ^ 1u);
-    const int t = threadIdx.x;
-    const int cl = blockIdx.x / 2, ncl = gridDim.x / 2;
-    auto src_rows = [&](int g) {   // first of this CTA's two rows of group g
-        const int item = g / groups_per_item, y0 = (g % groups_per_item) * 4 + 2 * (int)rank;
-        return in + item * in_item_stride + (long long)y0 * N;
+    const int r = threadIdx.x % R, t = threadIdx.x / R;
+    const float2* w = split_phase_of<P>(tw) + t;
+    const TwTable<Q> twt{tw, t};
+    float2 v[16];
+    auto load = [&](int g) {
+        const int item = g / groups_per_item, y = (g % groups_per_item) * R + r;
+        const float2* src = in + item * in_item_stride + (long long)y * Q + t;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = __ldg(src + e * T);
     };
-    auto issue = [&](int g) {
-        const float2* src = src_rows(g);
-        mbar_arrive_expect_tx(mbar, (unsigned)(2 * N * sizeof(float2)));
-        bulk_load(stage, src, (unsigned)(N * sizeof(float2)), mbar);
-        bulk_load(stage + SST, src + N, (unsigned)(N * sizeof(float2)), mbar);
-    };
-    if (threadIdx.x == 0) {
-        mbar_init(mbar, 1);
-        if (BULK && cl < total_groups) issue(cl);
-    }
-    __syncthreads();
-    unsigned parity = 0;
+    int g = blockIdx.x, h = 0;
+    if (g < total_groups) load(g);
 #pragma unroll 1
-    for (int g = cl; g < total_groups; g += ncl, parity ^= 1u) {
-        float2 a[16], b[16];
-        if constexpr (BULK) {
-            mbar_wait_bounded(mbar, parity, status);     // on expiry: status bit set, loop continues
-#pragma unroll
-            for (int e = 0; e < 8; ++e) { a[e] = stage[t + e * T]; b[e] = stage[SST + t + e * T]; }
-            fence_proxy_async_smem();
-        } else {
-            const float2* src = src_rows(g);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) { a[e] = __ldg(src + t + e * T); b[e] = __ldg(src + N + t + e * T); }
-        }
-#pragma unroll
-        for (int e = 8; e < 16; ++e) { a[e] = make_float2(0.f, 0.f); b[e] = make_float2(0.f, 0.f); }
+    while (g < total_groups) {
+        const int item = g / groups_per_item, y0 = (g % groups_per_item) * R;
         if constexpr (PRE) {
-            const int yr = (g % groups_per_item) * 4 + 2 * (int)rank;
-            const float2 fy0 = __ldg(pre.fy + yr), fy1 = __ldg(pre.fy + yr + 1);
+            const float2 fy = __ldg(pre.fy + y0 + r);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float2 fx = __ldg(pre.fx + t + e * T);
-                a[e] = cmul(a[e], cmul(fx, fy0));
-                b[e] = cmul(b[e], cmul(fx, fy1));
-            }
+            for (int e = 0; e < 16; ++e) v[e] = cmul(v[e], cmul(__ldg(pre.fx + t + e * T), fy));
         }
-        __syncthreads();
-        if (BULK && threadIdx.x == 0 && g + ncl < total_groups) issue(g + ncl);
-        stage_butterflies<P, 0, false, 8>(a);
-        stage_butterflies<P, 0, false, 8>(b);
-        twiddle2<P, 0, false>(a, b, tw, t);
-        if (threadIdx.x == 0) tma_store_wait_read();     // this CTA's previous tile read out
-        __syncthreads();
-        xch2v<P, 1, 0, 1>(sx, 0, t, a, b);
-        fwd2v_from<P, 1, 1, 8>(a, b, sx, 0, t, tw);
-        cluster_sync();   // both exchange regions free (every exchange read done); both previous tiles read out
+        if (h) {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {   // storage column e T + t lies in half e / 8; rows 2 rank, + 1
-            const int q = ((e & 7) * T + t) * 2 + (int)rank;   // float4 slot of the 4-row tile
-            const float4 w = make_float4(a[e].x, a[e].y, b[e].x, b[e].y);
-            if ((e >> 3) == (int)rank) sx[q] = w;
-            else st_cluster4(tile_remote + (unsigned)(q * sizeof(float4)), w);
+            for (int e = 0; e < 16; ++e) v[e] = cmul(v[e], __ldg(w + e * T));
         }
-        fence_proxy_async_cluster();
-        cluster_sync();   // every value of both tiles written
+        stage_butterflies<Q, 0, false, 16>(v);
+        twt.template apply<0, false>(v);
+        if (threadIdx.x == 0) tma_store_wait_read();   // the previous tile, which the exchange region aliases
+        __syncthreads();
+        xch1<Q, R, 0, 1>(sm, r, t, v);
+        fwd1_from<Q, R, 1, 16>(v, sm, r, t, twt);
+        __syncthreads();   // every exchange read done before the tile is written
+#pragma unroll
+        for (int e = 0; e < 16; ++e) sm[e * NT + threadIdx.x] = v[e];
+        const int half = h;
+        h ^= 1;
+        if (h == 0) g += gridDim.x;
+        if (g < total_groups) load(g);
+        fence_proxy_async_smem();
+        __syncthreads();
         if (threadIdx.x == 0) {
-            const int item = g / groups_per_item, y0 = (g % groups_per_item) * 4;
 #pragma unroll 1
-            for (int bb = 0; bb < HALF / BOX; ++bb)
-                tma_store_3d(&wmap, sm + bb * BOX * 4, y0, (int)rank * HALF + bb * BOX, item + item_off);
+            for (int b = 0; b < Q / BOX; ++b) tma_store_3d(&wmap, sm + b * BOX * R, y0, half * Q + b * BOX, item + item_off);
             tma_store_commit();
         }
     }
     if (threadIdx.x == 0) tma_store_wait_read();
-    cluster_sync();   // no CTA leaves while its partner may still use its shared memory
+}
+
+// Inverse: two tile buffers, one per half, each aliasing its exchange region.  A half's tile of the
+// next group is requested as soon as the half's last exchange has been read back, so it loads while
+// the other half is transformed; the even half's values wait in registers for the odd ones.
+template <int P, int R>
+__host__ __device__ constexpr size_t row_inv_s_smem_bytes() {
+    return 2 * row_smem_words<P / 2, R>() * sizeof(float2) + 2 * sizeof(uint64_t);
+}
+
+template <int P, int R, int EPI>
+__global__ void __launch_bounds__(R * (P / 32), 1)
+k_row_inv_s(const __grid_constant__ CUtensorMap wmap, int item_off, float2* __restrict__ out,
+            long long out_item_stride, int groups_per_item, int total_groups, float scale,
+            const float4* __restrict__ tw, int* status, const Epilogue ep) {
+    pdl_wait();
+    constexpr int Q = P / 2, T = Q / 16, NT = R * T, BOX = kTmaBoxCols;
+    constexpr size_t BUF = row_smem_words<Q, R>();
+    static_assert(BUF * sizeof(float2) % 128 == 0, "TMA destination");
+    extern __shared__ __align__(1024) float2 sm[];
+    uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + 2 * BUF);
+    const int r = threadIdx.x % R, t = threadIdx.x / R;
+    auto issue = [&](int g, int h) {   // thread 0: half h of the R-row tile of group g
+        const int item = g / groups_per_item, y0 = (g % groups_per_item) * R;
+        mbar_arrive_expect_tx(mbar + h, (unsigned)(R * Q * sizeof(float2)));
+#pragma unroll 1
+        for (int b = 0; b < Q / BOX; ++b)
+            tma_load_3d(sm + h * BUF + b * BOX * R, &wmap, mbar + h, y0, h * Q + b * BOX, item + item_off);
+    };
+    if (threadIdx.x == 0) {
+        mbar_init(mbar, 1);
+        mbar_init(mbar + 1, 1);
+        if ((int)blockIdx.x < total_groups) {
+            issue(blockIdx.x, 0);
+            issue(blockIdx.x, 1);
+        }
+    }
+    __syncthreads();
+    const TwTable<Q> twt{tw, t};
+    const float2* w = split_phase_of<P>(tw) + t;
+    unsigned parity = 0;
+    int h = 0;
+    float2 even[16];
+#pragma unroll 1
+    for (int g = blockIdx.x; g < total_groups;) {
+        const bool ok = mbar_wait_bounded(mbar + h, parity, status);
+        float2* buf = sm + h * BUF;
+        float2 v[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = buf[e * NT + threadIdx.x];
+        if (__syncthreads_or(!ok)) {   // a copy did not land: the status word says so
+            // the copies of the other half still in flight land (or give up) before the block leaves
+            if (h == 0 || g + (int)gridDim.x < total_groups) mbar_wait_bounded(mbar + (h ^ 1), h == 0 ? parity : parity ^ 1u, status);
+            break;
+        }
+        inv1_to_stage0<Q, R, Geo<Q>::NST - 1>(v, buf, r, t, twt);
+        fence_proxy_async_smem();      // the exchange reads precede the next tile load
+        __syncthreads();
+        if (threadIdx.x == 0 && g + (int)gridDim.x < total_groups) issue(g + gridDim.x, h);
+        twt.template apply<0, true>(v);
+        stage_butterflies<Q, 0, true, 16>(v);
+        if (h == 0) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) even[e] = v[e];
+        } else {
+            const int item = g / groups_per_item, y0 = (g % groups_per_item) * R;
+            const long long base = item * out_item_stride + (long long)(y0 + r) * Q;
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+                epilogue_store<EPI>(out, ep, base + t + e * T, t + e * T, y0 + r,
+                                    cscale(cadd(even[e], cmulc(v[e], __ldg(w + e * T))), scale));
+            g += gridDim.x;
+            parity ^= 1u;
+        }
+        h ^= 1;
+    }
 }
 
 // Inverse, persistent: R rows per group, one tile buffer.  The tile of the NEXT group is
@@ -361,77 +402,6 @@ k_row_inv_p(const __grid_constant__ CUtensorMap wmap, int item_off, float2* __re
         const long long base = item * out_item_stride + (long long)(y0 + r) * N;
 #pragma unroll
         for (int e = 0; e < 8; ++e) epilogue_store<EPI>(out, ep, base + t + e * T, t + e * T, y0 + r, cscale(v[e], scale));   // crop
-    }
-}
-
-
-
-// Inverse, pair form (P = 8192): each thread transforms two rows of the group (2 cp and 2 cp + 1
-// of its CP = R / 2 pairs), which share every twiddle load, and moves both rows' values at one
-// position with one 128-bit access -- in the tile read (the tile [st][r] holds the pair at
-// st R + 2 cp, + 1) and in the exchanges (PairLayout, one barrier each).  Otherwise as
-// k_row_inv_p: one tile buffer aliasing the exchange region, the next group's tile requested after
-// the last exchange.  Measured per field against k_row_inv_p: 4096^2 159.6 against 171.5 us; at
-// 2048^2 (24.2 against 23.0 us) and 1024^2 (5.85 against 5.70) the half as many warps per SM cost
-// more than the shared twiddle loads save.
-template <int P, int CP>
-__host__ __device__ constexpr size_t row_inv_pp_words() {
-    return 2 * (size_t)PairLayout<P, CP>::SLOTS > (size_t)2 * CP * P ? 2 * (size_t)PairLayout<P, CP>::SLOTS
-                                                                       : (size_t)2 * CP * P;
-}
-
-template <int P, int CP, int EPI>
-__global__ void __launch_bounds__(CP * (P / 16), CP * (P / 16) >= 512 ? 1 : 2)
-k_row_inv_pp(const __grid_constant__ CUtensorMap wmap, int item_off, float2* __restrict__ out,
-             long long out_item_stride, int groups_per_item, int total_groups, float scale,
-             const float4* __restrict__ tw, int* status, const Epilogue ep) {
-    pdl_wait();
-    constexpr int R = 2 * CP, T = P / 16, N = P / 2;
-    constexpr int BOX = P < kTmaBoxCols ? P : kTmaBoxCols;
-    static_assert(Geo<P>::NST >= 2 && P >= 128, "at least two stages, 128-bit pair exchanges");
-    extern __shared__ __align__(1024) float2 sm[];
-    float4* sx = reinterpret_cast<float4*>(sm);
-    const float4* tile = reinterpret_cast<const float4*>(sm);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + row_inv_pp_words<P, CP>());
-    const int t = CP == 1 ? (int)threadIdx.x : (int)threadIdx.x % T;
-    const int cp = CP == 1 ? 0 : (int)threadIdx.x / T;
-    auto issue = [&](int g) {   // thread 0: the R-row tile of group g
-        const int item = g / groups_per_item, y0 = (g % groups_per_item) * R;
-        mbar_arrive_expect_tx(mbar, (unsigned)(R * P * sizeof(float2)));
-#pragma unroll 1
-        for (int b = 0; b < P / BOX; ++b) tma_load_3d(sm + b * BOX * R, &wmap, mbar, y0, b * BOX, item + item_off);
-    };
-    if (threadIdx.x == 0) {
-        mbar_init(mbar, 1);
-        if ((int)blockIdx.x < total_groups) issue(blockIdx.x);
-    }
-    __syncthreads();
-    unsigned parity = 0;
-#pragma unroll 1
-    for (int g = blockIdx.x; g < total_groups; g += gridDim.x, parity ^= 1u) {
-        const bool ok = mbar_wait_bounded(mbar, parity, status);
-        float2 a[16], b[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const float4 q = tile[(e * T + t) * CP + cp];
-            a[e] = make_float2(q.x, q.y);
-            b[e] = make_float2(q.z, q.w);
-        }
-        if (__syncthreads_or(!ok)) break;          // a copy did not land: the status word says so
-        inv2v_to_stage0<P, CP, Geo<P>::NST - 1>(a, b, sx, cp, t, tw);
-        fence_proxy_async_smem();                  // the exchange reads precede the next tile load
-        __syncthreads();
-        if (threadIdx.x == 0 && g + (int)gridDim.x < total_groups) issue(g + gridDim.x);
-        twiddle2<P, 0, true>(a, b, tw, t);
-        stage_butterflies<P, 0, true, 16>(a);
-        stage_butterflies<P, 0, true, 16>(b);
-        const int item = g / groups_per_item, y0 = (g % groups_per_item) * R + 2 * cp;
-        const long long base = item * out_item_stride + (long long)y0 * N;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {   // crop: positions t + e T < N of rows y0 and y0 + 1
-            epilogue_store<EPI>(out, ep, base + t + e * T, t + e * T, y0, cscale(a[e], scale));
-            epilogue_store<EPI>(out, ep, base + N + t + e * T, t + e * T, y0 + 1, cscale(b[e], scale));
-        }
     }
 }
 
@@ -510,22 +480,6 @@ static cudaError_t row_turn_impl(const CUtensorMap* wmap, int ny, int items, lon
     }
 }
 
-template <int P, bool PRE, bool BULK>
-static cudaError_t row_fwd_c_launch(const float2* in, long long in_item_stride, const CUtensorMap* wmap, int item_off,
-                                    int ny, int items, const float4* tw, int* status, const Prefactor& pre,
-                                    cudaStream_t st) {
-    constexpr int T = P / 16;
-    const int groups = (ny / 4) * items;
-    int clusters = 0;
-    const size_t smem = row_fwd_c_smem_bytes<P>();
-    cudaError_t e = cluster_setup<k_row_fwd_c<P, PRE, BULK>>(smem, T, &clusters);
-    if (e != cudaSuccess) return e;
-    if (clusters < 1) return cudaErrorInvalidConfiguration;
-    const int grid = 2 * std::min(groups, clusters);
-    return pdl_launch(k_row_fwd_c<P, PRE, BULK>, dim3(grid), dim3(T), smem, st, in, in_item_stride, *wmap, item_off,
-                      ny / 4, groups, tw, status, pre);
-}
-
 template <int P, bool PRE>
 static cudaError_t row_fwd_impl_t(const float2* in, long long in_item_stride, const CUtensorMap* wmap,
                                   int item_off, int ny, int items, const float4* tw, int* status, const Prefactor& pre,
@@ -533,12 +487,19 @@ static cudaError_t row_fwd_impl_t(const float2* in, long long in_item_stride, co
     constexpr int R = rows_fwd<P>();
     constexpr int T = P / 16;
     if (ny % R) return cudaErrorInvalidValue;
+    if constexpr (P >= 8192) {
+        const size_t smem = row_smem_words<P / 2, R>() * sizeof(float2);
+        int resident = 0;
+        cudaError_t e = kernel_setup<k_row_fwd_s<P, R, PRE>>(smem, R * T / 2, &resident);
+        if (e != cudaSuccess) return e;
+        const int groups = (ny / R) * items;
+        const int grid = std::min(groups, resident);
+        if (grid < 1) return cudaErrorInvalidConfiguration;
+        return pdl_launch(k_row_fwd_s<P, R, PRE>, dim3(grid), dim3(R * T / 2), smem, st, in, in_item_stride, *wmap, item_off,
+                          ny / R, groups, tw, pre);
+    } else {
     // persistent pipelined kernel where its bulk copies are legal: rows start on 16-byte boundaries
     const bool aligned = ((uintptr_t)in % 16 == 0) && (in_item_stride % 2 == 0);
-    if constexpr (rows_fwd_cluster<P>()) {
-        return aligned ? row_fwd_c_launch<P, PRE, true>(in, in_item_stride, wmap, item_off, ny, items, tw, status, pre, st)
-                       : row_fwd_c_launch<P, PRE, false>(in, in_item_stride, wmap, item_off, ny, items, tw, status, pre, st);
-    } else {
     if (P >= 512 && aligned) {
         const size_t smem = row_fwd_p_smem_bytes<P, R>();
         int resident = 0;
@@ -578,18 +539,17 @@ static cudaError_t row_inv_impl_e(const CUtensorMap* wmap, int item_off, float2*
     constexpr int T = P / 16;
     const size_t smem = row_smem_words<P, R>() * sizeof(float2) + sizeof(uint64_t);   // tile + mbarrier
     if (ny % R) return cudaErrorInvalidValue;
-    if constexpr (P >= 8192 && R % 2 == 0) {
-        constexpr int CP = R / 2;
-        const size_t psmem = row_inv_pp_words<P, CP>() * sizeof(float2) + sizeof(uint64_t);
+    if constexpr (P >= 8192) {
+        const size_t ssmem = row_inv_s_smem_bytes<P, R>();
         int resident = 0;
-        cudaError_t e = kernel_setup<k_row_inv_pp<P, CP, EPI>>(psmem, CP * T, &resident);
+        cudaError_t e = kernel_setup<k_row_inv_s<P, R, EPI>>(ssmem, R * T / 2, &resident);
         if (e != cudaSuccess) return e;
         const int groups = (ny / R) * items;
         const int grid = std::min(groups, resident);
-        if (grid > 0)
-            return pdl_launch(k_row_inv_pp<P, CP, EPI>, dim3(grid), dim3(CP * T), psmem, st, *wmap, item_off, out,
-                              out_item_stride, ny / R, groups, scale, tw, status, ep);
-    }
+        if (grid < 1) return cudaErrorInvalidConfiguration;
+        return pdl_launch(k_row_inv_s<P, R, EPI>, dim3(grid), dim3(R * T / 2), ssmem, st, *wmap, item_off, out,
+                          out_item_stride, ny / R, groups, scale, tw, status, ep);
+    } else {
     if constexpr (kRowInvPersistent && P >= 512) {
         int resident = 0;
         cudaError_t e = kernel_setup<k_row_inv_p<P, R, EPI>>(smem, R * T, &resident);
@@ -606,6 +566,7 @@ static cudaError_t row_inv_impl_e(const CUtensorMap* wmap, int item_off, float2*
     dim3 grid(ny / R, items);
     return pdl_launch(k_row_inv<P, R, EPI>, grid, dim3(R * T), smem, st, *wmap, item_off, out, out_item_stride, scale, tw,
                       status, ep);
+    }
 }
 
 template <int P>

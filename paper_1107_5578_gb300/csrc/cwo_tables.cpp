@@ -28,17 +28,18 @@ int ilog2i(int n) { int l = 0; while ((1 << l) < n) ++l; return l; }
 
 double frac01(double x) { return x - std::floor(x); }
 
-AxisGeo::AxisGeo(int p) : P(p), T(p / 16) {
+AxisGeo::AxisGeo(int p, bool split_order) : P(p), T(p / 16), split(split_order) {
     const int lg = ilog2i(p);
     NST = (lg + 3) / 4;
     RLAST = 1 << (lg - 4 * (NST - 1));
 }
 
 // pos = sum_s k_s P / (r_0..r_s)  and  k = sum_s k_s (r_0..r_{s-1})
-int AxisGeo::freq_of_pos(int pos) const {
+namespace {
+int dif_freq(int P, int NST, int RLAST, int pos) {
     int k = 0, below = 1, above = P;
     for (int s = 0; s < NST; ++s) {
-        const int r = radix(s);
+        const int r = s == NST - 1 ? RLAST : 16;
         above /= r;
         const int ks = (pos / above) % r;
         k += ks * below;
@@ -46,8 +47,29 @@ int AxisGeo::freq_of_pos(int pos) const {
     }
     return k;
 }
+// one object per length, built on first use and never changed
+template <class T, class Make>
+const T& kept(std::mutex& mu, std::map<int, std::unique_ptr<T>>& all, int P, const Make& make) {
+    std::lock_guard<std::mutex> lk(mu);
+    auto& slot = all[P];
+    if (!slot) slot = std::make_unique<T>(make());
+    return *slot;
+}
+}  // namespace
 
-std::vector<float4> twiddle_table(const AxisGeo& g) {
+int AxisGeo::freq_of_pos(int pos) const { return dif_freq(P, NST, RLAST, pos); }
+
+int AxisGeo::freq_of_idx(int idx) const {
+    if (!split) return freq_of_pos(16 * (idx % T) + idx / T);
+    const int Q = P / 2, Tq = Q / 16, i = idx % Q;
+    int lg = 0;
+    while ((1 << lg) < Q) ++lg;
+    const int nst = (lg + 3) / 4;
+    return 2 * dif_freq(Q, nst, 1 << (lg - 4 * (nst - 1)), 16 * (i % Tq) + i / Tq) + idx / Q;
+}
+
+namespace {
+std::vector<float4> make_twiddles(const AxisGeo& g) {
     // per radix-16 stage s (all but the last): 8 S_s float4 laid out [kp][j], kp = 0..7,
     // j = 0..S_s-1 (= t mod S_s), holding (W_L^{j (2kp+1)}, W_L^{j (2kp+2)}), L = L_s
     std::vector<float4> tw((size_t)g.tw_off(g.NST - 1));
@@ -68,6 +90,13 @@ std::vector<float4> twiddle_table(const AxisGeo& g) {
     }
     return tw;
 }
+}  // namespace
+
+const std::vector<float4>& twiddle_table(const AxisGeo& g) {
+    static std::mutex mu;
+    static std::map<int, std::unique_ptr<std::vector<float4>>> all;
+    return kept(mu, all, g.P, [&] { return make_twiddles(g); });
+}
 
 std::vector<int2> mirror_pairs(const AxisGeo& g) {
     std::vector<int> where(g.P);
@@ -84,25 +113,29 @@ std::vector<int> bin_table(const AxisGeo& g) {
     return b;
 }
 
-std::vector<int> split_axis_index(int P) {
-    const AxisGeo g(P), gq(P / 2);
-    std::vector<int> where(P);
-    for (int i = 0; i < P; ++i) where[g.freq_of_idx(i)] = i;
-    std::vector<int> out(P);
-    for (int i = 0; i < P; ++i) {
-        const int h = i / gq.P, idx = i % gq.P;
-        out[i] = where[2 * gq.freq_of_idx(idx) + h];
-    }
-    return out;
+const std::vector<int>& split_axis_index(int P) {
+    static std::mutex mu;
+    static std::map<int, std::unique_ptr<std::vector<int>>> all;
+    return kept(mu, all, P, [&] {
+        const AxisGeo g(P), gs(P, true);
+        std::vector<int> where(P), out(P);
+        for (int i = 0; i < P; ++i) where[g.freq_of_idx(i)] = i;
+        for (int i = 0; i < P; ++i) out[i] = where[gs.freq_of_idx(i)];
+        return out;
+    });
 }
 
-std::vector<float2> split_phase(int P) {
-    std::vector<float2> w(P / 2);
-    for (int n = 0; n < P / 2; ++n) {
-        const double ang = -2.0 * kPi * (double)n / (double)P;
-        w[n] = make_float2((float)std::cos(ang), (float)std::sin(ang));
-    }
-    return w;
+const std::vector<float2>& split_phase(int P) {
+    static std::mutex mu;
+    static std::map<int, std::unique_ptr<std::vector<float2>>> all;
+    return kept(mu, all, P, [&] {
+        std::vector<float2> w(P / 2);
+        for (int n = 0; n < P / 2; ++n) {
+            const double ang = -2.0 * kPi * (double)n / (double)P;
+            w[n] = make_float2((float)std::cos(ang), (float)std::sin(ang));
+        }
+        return w;
+    });
 }
 
 // Per-length caches: twiddles W_P^j (j < P/2) of the FP64 FFT, and the axis-index lists of the
@@ -114,11 +147,11 @@ struct AxisCache {
     std::vector<int> first, second;      // for |k| = 0 .. P/2: the axis indices of +k and -k
 };
 std::mutex g_cache_mu;
-std::map<int, std::unique_ptr<AxisCache>> g_cache;
+std::map<std::pair<int, bool>, std::unique_ptr<AxisCache>> g_cache;
 
-const AxisCache& axis_cache(int P) {
+const AxisCache& axis_cache(int P, bool split = false) {
     std::lock_guard<std::mutex> lk(g_cache_mu);
-    auto& slot = g_cache[P];
+    auto& slot = g_cache[{P, split}];
     if (!slot) {
         auto c = std::make_unique<AxisCache>();
         c->wre.resize(P / 2);
@@ -128,7 +161,7 @@ const AxisCache& axis_cache(int P) {
             c->wre[j] = std::cos(ang);
             c->wim[j] = std::sin(ang);
         }
-        const AxisGeo g(P);
+        const AxisGeo g(P, split);
         c->kabs.resize(P);
         c->first.assign(P / 2 + 1, -1);
         c->second.assign(P / 2 + 1, -1);
@@ -266,7 +299,7 @@ AsmAxis asm_axis(int P, double pitch, double lambda, double z, bool is_x) {
 void asm_axis_table(const AxisGeo& g, double pitch, double lambda, double z, bool is_x, float4* out) {
     const AsmAxis A = asm_axis(g.P, pitch, lambda, z, is_x);
     // every entry depends on kt^2 only: evaluate |kt| = 0 .. P/2 once, store at both indices
-    const AxisCache& c = axis_cache(g.P);
+    const AxisCache& c = axis_cache(g.P, g.split);
     for (int k = 0; k <= g.P / 2; ++k) {
         const float4 v = asm_axis_entry(A, (double)k * (double)k);
         out[c.first[k]] = v;
@@ -326,7 +359,7 @@ float2 unit_cycles(double cyc) {
 }  // namespace
 
 void shifted_fresnel_axis(int n, double p0, double p1, double o0, double o1, double lambda, double z, cd coeff,
-                          float2* f, float2* q, float2* h) {
+                          float2* f, float2* q, float2* h, bool split) {
     const double lz = lambda * z;
     const double S = p0 * p1 / lz;
     for (int a = 0; a < n; ++a) {
@@ -346,7 +379,7 @@ void shifted_fresnel_axis(int n, double p0, double p1, double o0, double o1, dou
         if (d > 0 && d < P / 2) hd[P - d] = hd[d];
     }
     fft64(hd);
-    const AxisCache& c = axis_cache(P);
+    const AxisCache& c = axis_cache(P, split);
     for (int i = 0; i < P; ++i) {
         const cd v = hd[c.kabs[i]];
         h[i] = make_float2((float)v.real(), (float)v.imag());
@@ -402,8 +435,8 @@ int asm_tail_mode(int px, int py, double dx, double dy, double lambda, double z)
 }
 
 void make_h_tables(int px, int py, double dx, double dy, double lambda, double z, bool fresnel,
-                   bool literal_scale, float4* ax, float4* ay, float2* hx, float2* hy, float* kf) {
-    const AxisGeo gx(px), gy(py);
+                   bool literal_scale, float4* ax, float4* ay, float2* hx, float2* hy, float* kf, bool xsplit) {
+    const AxisGeo gx(px, xsplit), gy(py);
     if (!fresnel) {
         asm_axis_table(gx, dx, lambda, z, true, ax);
         asm_axis_table(gy, dy, lambda, z, false, ay);
@@ -420,7 +453,7 @@ void make_h_tables(int px, int py, double dx, double dy, double lambda, double z
         // frequencies are walked in natural order and each value is written to the axis indices
         // of +k and -k (reading H in the digit-reversed index order missed the cache on every
         // element: ~10 ns each at P = 8192)
-        const AxisCache& cx = axis_cache(px);
+        const AxisCache& cx = axis_cache(px, xsplit);
         for (int k = 0; k <= px / 2; ++k) {
             const cd h = Hx[k];
             const float2 v = make_float2((float)(cr * h.real() - ci * h.imag()), (float)(cr * h.imag() + ci * h.real()));

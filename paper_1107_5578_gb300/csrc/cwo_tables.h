@@ -13,21 +13,26 @@ namespace host {
 using cd = std::complex<double>;
 
 // Axis geometry, mirrored from the device FFT (cwo_fft.cuh): T = P/16 threads, stages of radix
-// 16 followed by one stage of radix RLAST.  Axis index idx = e*T + t <-> DIF position 16 t + e.
+// 16 followed by one stage of radix RLAST.  Axis index idx = e*T + t <-> DIF position 16 t + e, or,
+// split (the row passes at P = 8192; see split_axis_index), idx = h P/2 + i <-> frequency
+// 2 k + h, k the frequency of axis index i of the P/2-point transform.
 struct AxisGeo {
     int P, T, NST, RLAST;
-    explicit AxisGeo(int p);
+    bool split;
+    explicit AxisGeo(int p, bool split_order = false);
     int radix(int s) const { return s == NST - 1 ? RLAST : 16; }
     int len(int s) const { return P >> (4 * s); }
     int stride(int s) const { return len(s) / radix(s); }
     int tw_off(int s) const { return s <= 0 ? 0 : tw_off(s - 1) + 8 * stride(s - 1); }   // float4 units
     int freq_of_pos(int pos) const;   // bin whose forward DIF output lands at position pos
-    int freq_of_idx(int idx) const { return freq_of_pos(16 * (idx % T) + idx / T); }
+    int freq_of_idx(int idx) const;
     int signed_bin(int k) const { return k < P / 2 ? k : k - P; }
 };
 
 double frac01(double x);
-std::vector<float4> twiddle_table(const AxisGeo& g);
+// (kept per length for the life of the process, as are the split tables: thousands of FP64 sines that
+// every plan of a length would otherwise form again)
+const std::vector<float4>& twiddle_table(const AxisGeo& g);
 std::vector<int> bin_table(const AxisGeo& g);
 // storage columns of the frequencies +k and -k for k = 0 .. P/2 (0 and P/2 pair with themselves)
 std::vector<int2> mirror_pairs(const AxisGeo& g);
@@ -36,8 +41,8 @@ std::vector<int2> mirror_pairs(const AxisGeo& g);
 // i = h Q + idx (h = 0 even, 1 odd; idx a Q-point axis index) holds frequency 2 k(idx) + h.
 //   split_axis_index[i]: the P-point axis index (AxisGeo(P)) of the frequency at split index i
 //   split_phase[n]:      W_P^n for n < Q, correctly rounded from FP64
-std::vector<int> split_axis_index(int P);
-std::vector<float2> split_phase(int P);
+const std::vector<int>& split_axis_index(int P);
+const std::vector<float2>& split_phase(int P);
 void fft64(std::vector<cd>& x);
 std::vector<cd> fresnel_axis_dft(int P, double pitch, double lambda, double z);
 cd fresnel_coeff(double dx, double dy, double lambda, double z, bool literal_scale);
@@ -85,7 +90,7 @@ double band_limit_freq(int p, double pitch, double lambda, double z);
 //          index i (DIF order), made exactly even
 // phases reduced modulo one cycle in FP64; coeff multiplies q (pass 1 for the y axis).
 void shifted_fresnel_axis(int n, double p0, double p1, double o0, double o1, double lambda, double z, cd coeff,
-                          float2* f, float2* q, float2* h);
+                          float2* f, float2* q, float2* h, bool split = false);
 void fourier_tables(int nx, int ny, double dx, double dy, double lambda, double z, bool literal_scale,
                     float2* pre_x, float2* pre_y, float2* post_x, float2* post_y, int* st_of_col, int* row_of_idx);
 
@@ -102,7 +107,7 @@ struct HTables {
 int asm_tail_mode(int px, int py, double dx, double dy, double lambda, double z);
 
 void make_h_tables(int px, int py, double dx, double dy, double lambda, double z, bool fresnel,
-                   bool literal_scale, float4* ax, float4* ay, float2* hx, float2* hy, float* kf);
+                   bool literal_scale, float4* ax, float4* ay, float2* hx, float2* hy, float* kf, bool xsplit = false);
 
 }  // namespace host
 }  // namespace cwo
