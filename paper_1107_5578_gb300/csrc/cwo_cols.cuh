@@ -28,16 +28,28 @@
 
 namespace cwo {
 
-// columns per block (single-column kernel) and mirror pairs per block (paired kernel)
+// Columns per block (single-column kernel) and mirror pairs per block (paired kernel): as few as fill two
+// warps, so that the CTAs of an SM, which wait at their own barriers only, are many and a grid spreads
+// evenly over the SMs.  Measured against 256 threads per CTA, column pass: 64 512^2 fields 241 -> 237
+// us (cached transfer function 209 -> 203), 64 256^2 fields 67.6 -> 63.5, one 1024^2 field 22.5 -> 20.5
+// (513 CTAs on 304 places took two rounds).
 template <int P> constexpr int cols_per_block() {
     constexpr int T = P / 16;
-    constexpr int c = 256 / T;
+    constexpr int c = 64 / T;
     return c < 1 ? 1 : (c > 16 ? 16 : c);
 }
-template <int P> constexpr int col_min_blocks() { return (P / 16) * cols_per_block<P>() <= 256 ? 2 : 1; }
-// The paired kernel holds 32 values per thread (128 registers): two 256-thread CTAs per SM up to
-// P = 4096, one 512-thread CTA at P = 8192 (measured 382 us per 4096^2 field vs 488 for the
-// single-column kernel).  Single column per transform: plans whose H is not even in kx.
+// The paired kernel holds 32 values per thread (128 registers, 512 threads per SM), the shared-source
+// stack as many; the single-column kernel holds 16 and runs 768 threads per SM up to P = 4096: it
+// then spills a few words at 80 registers, and its column pass takes 197 us for 3 fields of 4096 x 1024
+// against 207 at 512 threads per SM and 199 at 1024 (2048^2, 4 fields: 294, 317, 290).
+template <int P, int C = cols_per_block<P>()> constexpr int colp_min_blocks() {
+    constexpr int n = 512 / (C * (P / 16));
+    return n < 1 ? 1 : n;
+}
+template <int P> constexpr int col_min_blocks() {
+    constexpr int n = (P <= 4096 ? 768 : 512) / (cols_per_block<P>() * (P / 16));
+    return n < 1 ? 1 : n;
+}
 template <int P, int C, bool MIXED>
 __global__ void __launch_bounds__(C * (P / 16), col_min_blocks<P>())
 k_col(const float2* __restrict__ win, long long win_item_stride, float2* __restrict__ wout,
@@ -82,7 +94,7 @@ constexpr int colp_smem_words() {
 }
 
 template <int P, int CP, bool MIXED>
-__global__ void __launch_bounds__(CP * (P / 16), CP * (P / 16) >= 512 ? 1 : 2)
+__global__ void __launch_bounds__(CP * (P / 16), colp_min_blocks<P, CP>())
 k_colp(const float2* __restrict__ win, long long win_item_stride, float2* __restrict__ wout,
        long long wout_item_stride, const float4* __restrict__ tw, const HParams hp, int resident) {
     pdl_wait();
@@ -221,7 +233,7 @@ k_col_split(const float2* __restrict__ win, long long win_item_stride, float2* _
 // transforms it back and writes the plane (Section "Three-dimensional diffraction calculations":
 // a stack of 2-D diffractions of one source).
 template <int P, int C>
-__global__ void __launch_bounds__(C * (P / 16), col_min_blocks<P>())
+__global__ void __launch_bounds__(C * (P / 16), colp_min_blocks<P>())
 k_col_stack(const float2* __restrict__ win, float2* __restrict__ wout, long long wout_item_stride, int nplanes,
             const float4* __restrict__ tw, const HParams hp) {
     pdl_wait();
@@ -253,6 +265,19 @@ k_col_stack(const float2* __restrict__ win, float2* __restrict__ wout, long long
 }
 
 
+template <int P, int CP, bool MIXED>
+static cudaError_t colp_launch(const float2* win, long long win_item_stride, float2* wout, long long wout_item_stride,
+                               int items, const float4* tw, const HParams& hp, cudaStream_t st) {
+    constexpr int T = P / 16;
+    const size_t smem = (size_t)colp_smem_words<P, CP>() * sizeof(float2);
+    int resident = 0;
+    cudaError_t e = kernel_setup<k_colp<P, CP, MIXED>>(smem, CP * T, &resident);
+    if (e != cudaSuccess) return e;
+    const unsigned blocks = (unsigned)((hp.npairs + CP - 1) / CP);
+    return pdl_launch(k_colp<P, CP, MIXED>, dim3(items, blocks), dim3(CP * T), smem, st, win, win_item_stride, wout,
+                      wout_item_stride, tw, hp, resident);
+}
+
 template <int P, bool MIXED>
 static cudaError_t col_impl_t(const float2* win, long long win_item_stride, float2* wout,
                               long long wout_item_stride, int px, int items, const float4* tw,
@@ -281,15 +306,16 @@ static cudaError_t col_impl_t(const float2* win, long long win_item_stride, floa
                        wout_item_stride, tw, hp);
         if (e != cudaSuccess) return e;
     } else {         // H even in kx: mirror pairs
-        constexpr int CP = cols_per_block<P>();
         if (hp.npairs != px / 2 + 1 || !hp.pairs) return cudaErrorInvalidValue;
-        const size_t smem = (size_t)colp_smem_words<P, CP>() * sizeof(float2);
-        int resident = 0;
-        if ((e = kernel_setup<k_colp<P, CP, MIXED>>(smem, CP * T, &resident))) return e;
-        const unsigned blocks = (unsigned)((hp.npairs + CP - 1) / CP);
-        e = pdl_launch(k_colp<P, CP, MIXED>, dim3(items, blocks), dim3(CP * T), smem, st, win, win_item_stride, wout,
-                       wout_item_stride, tw, hp, resident);
-        if (e != cudaSuccess) return e;
+        // two pairs per CTA at P = 2048 for a batch that evaluates H per element: the CTA's pairs share the
+        // item's y table in L1 (7 1024^2 fields with their own distances 112.4 us against 114.2 for one
+        // pair; cached, 16 fields, 219 against 216)
+        constexpr int CP = cols_per_block<P>();
+        if constexpr (P == 2048) {
+            if (hp.mode != HMODE_TABLE && items >= 4)
+                return colp_launch<P, 2 * CP, MIXED>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);
+        }
+        return colp_launch<P, CP, MIXED>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);
     }
     return cudaGetLastError();
 }
