@@ -16,17 +16,15 @@ namespace cwo {
 // and is launched with programmatic stream serialisation, so its launch is processed while the
 // previous grid runs.  No kernel triggers its dependents early (griddepcontrol.launch_dependents):
 // measured on GB300, every placement of the trigger cost time (up to 2 us per 2048^2 field) or
-// gained nothing, while the launch overlap alone takes 512^2 propagations from 22.6 to 15.2 us.
+// gained nothing, while the launch overlap alone takes 512^2 propagations from 22.6 to 15.2 us.  Grids of
+// many waves gain the same few microseconds between passes (64 512^2 fields, Fresnel: 210.0 -> 205.6
+// us, angular spectrum 396 -> 393), so none is launched plainly.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// grids of more CTAs than this are launched plainly (many waves: nothing to overlap)
-constexpr unsigned kPdlMaxCtas = 4096;
 
 template <typename... KArgs, typename... Args>
 cudaError_t pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
-    const bool pdl = (unsigned long long)grid.x * grid.y * grid.z <= kPdlMaxCtas;
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
@@ -35,7 +33,7 @@ cudaError_t pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 #endif
