@@ -297,7 +297,8 @@ cwo_status cwo_hologram_phase_grad(const void* g_c64, const float* phase, int h,
                                    float* gphase, void* cuda_stream);
 
 /* Number of kernel launches one call of cwo_propagate_batch makes for this plan (for launch
- * accounting in benchmarks): 3 for the angular spectrum types, 2 for the Fresnel Fourier form and
+ * accounting in benchmarks): 3 for the angular spectrum types (one more for a large batch of small
+ * fields, whose transfer function is evaluated once for all of them), 2 for the Fresnel Fourier form and
  * for the Fresnel convolution and shifted Fresnel types, whose separable line passes take 2 (3
  * for an output epilogue, an output or a stack source not on a 16-byte boundary, a shifted
  * Fresnel z-stack, or a z-stack of padded rows longer than 4096). */

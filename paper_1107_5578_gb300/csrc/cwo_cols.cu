@@ -6,6 +6,7 @@
 namespace cwo {
 
 __global__ void k_build_hcache(float2* __restrict__ out, int py, const HParams hp, const int* __restrict__ yidx) {
+    pdl_wait();   // the previous call's column pass may still read the table
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
     if (o >= py) return;
@@ -21,8 +22,7 @@ __global__ void k_build_hcache(float2* __restrict__ out, int py, const HParams h
 
 cudaError_t launch_build_hcache(float2* out, int npairs, int py, const HParams& hp, cudaStream_t st, const int* yidx) {
     if (npairs < 1 || py < 1 || hp.mode > HMODE_ASM_FP64) return cudaErrorInvalidValue;
-    k_build_hcache<<<dim3((unsigned)((py + 255) / 256), (unsigned)npairs), 256, 0, st>>>(out, py, hp, yidx);
-    return cudaGetLastError();
+    return pdl_launch(k_build_hcache, dim3((unsigned)((py + 255) / 256), (unsigned)npairs), dim3(256), 0, st, out, py, hp, yidx);
 }
 
 cudaError_t launch_col_stack(int py, const float2* win, float2* wout, long long wout_item_stride, int px, int planes,
