@@ -202,6 +202,17 @@ cwo_status cwo_propagate(cwo_plan* plan, const void* in_c64, void* out_c64, void
 cwo_status cwo_propagate_batch(cwo_plan* plan, const void* in, long long in_batch_stride,
                                void* out, int batch, const double* z_or_null, void* cuda_stream);
 
+/* One propagation (or, adjoint != 0, its adjoint) of a field of which only the rows [in_lo, in_hi) can be
+ * non-zero and only the rows [out_lo, out_hi) of the result are wanted: the other rows are neither
+ * transformed, read nor written.  Windows are widened to whole groups of cwo_propagate_rows_group(plan)
+ * rows: input rows of a touched group are read (and must hold their values, zeros outside the window),
+ * output rows of a touched group are written.  in and out may alias.  Angular spectrum plans
+ * (CWO_ANGULAR, but not with a cached transfer function at Ny = 4096): cwo_propagate_rows_group is the
+ * group size, 0 for plans that do not provide this call (CWO_ERR_UNSUPPORTED). */
+cwo_status cwo_propagate_rows(cwo_plan* plan, const void* in_c64, void* out_c64, int in_lo, int in_hi, int out_lo,
+                              int out_hi, int adjoint, void* cuda_stream);
+int cwo_propagate_rows_group(const cwo_plan* plan);
+
 /* One item of a mixed batch: its own diffraction type and parameters (same Nx x Ny as the plan). */
 typedef struct {
     double z;         /* distance, metres (non-zero for CWO_FRESNEL_CONV)           */
@@ -270,31 +281,25 @@ cwo_status cwo_propagate_epilogue(cwo_plan* plan, const void* in_c64, void* out_
 cwo_status cwo_gs_run(cwo_plan* plan, const float* amplitude, void* field_c64, float* intensity, int batch,
                       int iterations, void* cuda_stream);
 
-/* The steps of a phase-only hologram optimisation around a propagation and its adjoint.  A phase
- * [h][w] fills the window at column ox and row oy of an nx x ny canvas (any position and size inside
- * it; nx even, nx, ny <= CWO_MAX_SIDE); every buffer is contiguous device memory of the current device
- * owned by the caller, canvases complex64 [ny][nx], windows float [h][w]; canvases that are written
- * start on a 16-byte boundary.  All are enqueued on cuda_stream.
- *   field       field = exp(i phase) on the window, 0 elsewhere
- *   intensity   |u|^2 on the window
- *   loss        residual = |u|^2 - target on the window, loss = mean of its squares, summed in FP64 in a
- *               fixed order; partial: CWO_HOLOGRAM_PARTIALS doubles of scratch
- *   seed        2 u g s on the window, 0 elsewhere: with s = 1 (gloss NULL) the derivative by u
- *               (conjugate Wirtinger, as torch.autograd) of a loss whose derivative by |u|^2 is g; with
- *               gloss (one device float) s = 2 gloss / (h w), for g the residual above
- *   phase_grad  Re(conj(g) i exp(i phase)) on the window: the derivative by the phase of a loss
- *               whose derivative by the field is g */
+/* A phase-only hologram and the gradient of a loss of its reconstruction.  A phase [h][w] fills the window
+ * at column ox and row oy of the plan's Nx x Ny canvas (any position and size inside it):
+ *   forward    u = A exp(i phase), 0 outside the window before the propagation (the window's rows of u
+ *              are what backward and the outputs need; the others may stay unwritten).  Without a target
+ *              image = |u|^2 on the window; with one image = |u|^2 - target and loss = the mean of its
+ *              squares, summed in a fixed order, across threads in FP64 (partial: CWO_HOLOGRAM_PARTIALS doubles of
+ *              scratch)
+ *   backward   gphase = Re(conj(A^H (2 u g s)) i exp(i phase)) on the window: the derivative by the phase
+ *              of a loss whose derivative by |u|^2 is g s, with s = 1 (gloss NULL), or s = 2 gloss / (h w)
+ *              for g the residual above and gloss (one device float) the derivative by the loss
+ * Every buffer is contiguous device memory of the plan's device owned by the caller: u and work complex64
+ * [ny][nx] from a 16-byte boundary, the windows float [h][w].  Enqueued on cuda_stream; plans as
+ * for cwo_propagate and its adjoint (rows outside the window are left out where cwo_propagate_rows is
+ * provided). */
 #define CWO_HOLOGRAM_PARTIALS 1216
-cwo_status cwo_hologram_field(const float* phase, int h, int w, int nx, int ny, int ox, int oy, void* field_c64,
-                              void* cuda_stream);
-cwo_status cwo_hologram_intensity(const void* u_c64, int h, int w, int nx, int ny, int ox, int oy, float* intensity,
-                                  void* cuda_stream);
-cwo_status cwo_hologram_loss(const void* u_c64, const float* target, int h, int w, int nx, int ny, int ox, int oy,
-                             float* residual, float* loss, double* partial, void* cuda_stream);
-cwo_status cwo_hologram_seed(const void* u_c64, const float* g, const float* gloss, int h, int w, int nx, int ny, int ox,
-                             int oy, void* out_c64, void* cuda_stream);
-cwo_status cwo_hologram_phase_grad(const void* g_c64, const float* phase, int h, int w, int nx, int ny, int ox, int oy,
-                                   float* gphase, void* cuda_stream);
+cwo_status cwo_hologram_forward(cwo_plan* plan, const float* phase, const float* target, int h, int w, int ox, int oy,
+                                void* u_c64, float* image, float* loss, double* partial, void* cuda_stream);
+cwo_status cwo_hologram_backward(cwo_plan* plan, const float* phase, const void* u_c64, const float* g, const float* gloss,
+                                 int h, int w, int ox, int oy, void* work_c64, float* gphase, void* cuda_stream);
 
 /* Number of kernel launches one call of cwo_propagate_batch makes for this plan (for launch
  * accounting in benchmarks): 3 for the angular spectrum types (one more for a large batch of small

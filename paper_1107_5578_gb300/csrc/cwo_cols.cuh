@@ -93,7 +93,10 @@ constexpr int colp_smem_words() {
     return P >= 128 ? 2 * PairLayout<P, CP>::SLOTS : PadLayout<P, 2 * CP>::WORDS;
 }
 
-template <int P, int CP, bool MIXED>
+//
+// WIN: only the rows [hp.ylo, hp.yhi) of the columns are not zero (the others are not read), and only the
+// rows [hp.olo, hp.ohi) are stored; both bounds even.
+template <int P, int CP, bool MIXED, bool WIN = false>
 __global__ void __launch_bounds__(CP * (P / 16), colp_min_blocks<P, CP>())
 k_colp(const float2* __restrict__ win, long long win_item_stride, float2* __restrict__ wout,
        long long wout_item_stride, const float4* __restrict__ tw, const HParams hp, int resident) {
@@ -120,12 +123,13 @@ k_colp(const float2* __restrict__ win, long long win_item_stride, float2* __rest
                 const int jn = gn * CP + c;
                 if (jn >= hp.npairs) break;
                 const int2 pn = __ldg(hp.pairs + jn);
-                const float2* p0 = win + itn * win_item_stride + (long long)pn.x * NY;
-                const float2* p1 = win + itn * win_item_stride + (long long)pn.y * NY;
+                const int first = WIN ? hp.ylo : 0, bytes = 8 * (WIN ? hp.yhi - hp.ylo : NY);
+                const float2* p0 = win + itn * win_item_stride + (long long)pn.x * NY + first;
+                const float2* p1 = win + itn * win_item_stride + (long long)pn.y * NY + first;
                 if ((((uintptr_t)p0 | (uintptr_t)p1) & 15) == 0) {
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p0), "r"(NY * 8) : "memory");
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p0), "r"(bytes) : "memory");
                     if (pn.y != pn.x)
-                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p1), "r"(NY * 8) : "memory");
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p1), "r"(bytes) : "memory");
                 }
             }
         }
@@ -138,7 +142,14 @@ k_colp(const float2* __restrict__ win, long long win_item_stride, float2* __rest
     const float2* sb = win + item * win_item_stride + (long long)pr.y * NY;
     float2 a[16], b[16];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) { a[e] = __ldcg(sa + t + e * T); b[e] = __ldcg(sb + t + e * T); }
+    for (int e = 0; e < 8; ++e) {
+        if (WIN && (t + e * T < hp.ylo || t + e * T >= hp.yhi)) {
+            a[e] = b[e] = make_float2(0.f, 0.f);
+        } else {
+            a[e] = __ldcg(sa + t + e * T);
+            b[e] = __ldcg(sb + t + e * T);
+        }
+    }
 #pragma unroll
     for (int e = 8; e < 16; ++e) { a[e] = make_float2(0.f, 0.f); b[e] = make_float2(0.f, 0.f); }
     if constexpr (P >= 128) {
@@ -154,11 +165,13 @@ k_colp(const float2* __restrict__ win, long long win_item_stride, float2* __rest
     if (live) {
         float2* da = wout + item * wout_item_stride + (long long)pr.x * NY;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) da[t + e * T] = a[e];
+        for (int e = 0; e < 8; ++e)
+            if (!WIN || (t + e * T >= hp.olo && t + e * T < hp.ohi)) da[t + e * T] = a[e];
         if (pr.y != pr.x) {
             float2* db = wout + item * wout_item_stride + (long long)pr.y * NY;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) db[t + e * T] = b[e];
+            for (int e = 0; e < 8; ++e)
+                if (!WIN || (t + e * T >= hp.olo && t + e * T < hp.ohi)) db[t + e * T] = b[e];
         }
     }
 }
@@ -265,16 +278,16 @@ k_col_stack(const float2* __restrict__ win, float2* __restrict__ wout, long long
 }
 
 
-template <int P, int CP, bool MIXED>
+template <int P, int CP, bool MIXED, bool WIN = false>
 static cudaError_t colp_launch(const float2* win, long long win_item_stride, float2* wout, long long wout_item_stride,
                                int items, const float4* tw, const HParams& hp, cudaStream_t st) {
     constexpr int T = P / 16;
     const size_t smem = (size_t)colp_smem_words<P, CP>() * sizeof(float2);
     int resident = 0;
-    cudaError_t e = kernel_setup<k_colp<P, CP, MIXED>>(smem, CP * T, &resident);
+    cudaError_t e = kernel_setup<k_colp<P, CP, MIXED, WIN>>(smem, CP * T, &resident);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((hp.npairs + CP - 1) / CP);
-    return pdl_launch(k_colp<P, CP, MIXED>, dim3(items, blocks), dim3(CP * T), smem, st, win, win_item_stride, wout,
+    return pdl_launch(k_colp<P, CP, MIXED, WIN>, dim3(items, blocks), dim3(CP * T), smem, st, win, win_item_stride, wout,
                       wout_item_stride, tw, hp, resident);
 }
 
@@ -286,6 +299,7 @@ static cudaError_t col_impl_t(const float2* win, long long win_item_stride, floa
     cudaError_t e;
     if constexpr (P == kSplitColP && !MIXED) {
         if (hp.mode == HMODE_TABLE) {   // the cached H is stored in the split order at this Py
+            if (hp.win) return cudaErrorInvalidValue;
             if (hp.asym || !hp.split_tw || !hp.split_w || !hp.hcache || !hp.pairs || hp.npairs != px / 2 + 1)
                 return cudaErrorInvalidValue;
             const size_t smem = (size_t)colp_smem_words<P / 2, 1>() * sizeof(float2);
@@ -299,7 +313,7 @@ static cudaError_t col_impl_t(const float2* win, long long win_item_stride, floa
     }
     if (hp.asym) {   // H(kx) != H(-kx): one column per transform
         constexpr int C = cols_per_block<P>();
-        if (px % C != 0) return cudaErrorInvalidValue;
+        if (hp.win || px % C != 0) return cudaErrorInvalidValue;
         const size_t smem = (size_t)PadLayout<P, C>::WORDS * sizeof(float2);
         if ((e = kernel_setup<k_col<P, C, MIXED>>(smem, C * T, nullptr))) return e;
         e = pdl_launch(k_col<P, C, MIXED>, dim3(px / C, items), dim3(C * T), smem, st, win, win_item_stride, wout,
@@ -311,6 +325,9 @@ static cudaError_t col_impl_t(const float2* win, long long win_item_stride, floa
         // item's y table in L1 (7 1024^2 fields with their own distances 112.4 us against 114.2 for one
         // pair; cached, 16 fields, 219 against 216)
         constexpr int CP = cols_per_block<P>();
+        if constexpr (!MIXED) {
+            if (hp.win) return colp_launch<P, CP, false, true>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);
+        }
         if constexpr (P == 2048) {
             if (hp.mode != HMODE_TABLE && items >= 4)
                 return colp_launch<P, 2 * CP, MIXED>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);

@@ -7,6 +7,8 @@
 
 #include "cwo_tables.h"
 
+struct cwo_plan;
+
 namespace cwo {
 
 enum HMode : int {
@@ -87,6 +89,9 @@ struct HParams {
     // holds frequency 2 k + h, k the 4096-point frequency of register e of thread t)
     const float4* split_tw;
     const float2* split_w;
+    // win: rows [ylo, yhi) of the columns are read (the others are zero), rows [olo, ohi) stored
+    int win;
+    int ylo, yhi, olo, ohi;
 };
 
 // launchers (return cudaGetLastError() after the launch)
@@ -95,6 +100,9 @@ void set_last_error(const char* msg);
 // Check that [ptr, ptr + bytes) is `align`-byte aligned device (or managed) memory of `device` inside
 // one allocation (cuMemGetAddressRange); returns a cwo_status and sets the error message.
 int check_device_buffer(const void* ptr, size_t bytes, int device, const char* name, int align = 8);
+
+// the plan's Nx and Ny; false for a null plan
+bool plan_size(const ::cwo_plan* plan, int* nx, int* ny);
 
 // The intermediate is column-major: [items][Px][Ny] complex64 (see cwo_rows.cu).
 // The row passes reach the intermediate through rank-3 TMA tensor maps (Ny, Px, items) with
@@ -176,7 +184,8 @@ struct CopyList {
 };
 cudaError_t launch_copy_fields(const CopyList& list, int fields, long long elems, cudaStream_t st);
 // Encode the tensor map of an intermediate [cap][px][ny] at base (host only; no allocation).
-cudaError_t make_intermediate_map(CUtensorMap* map, void* base, int ny, int px, int cap, int rows);
+// window > 0: a map of `window` rows only, from the row that base points to (cap 1).
+cudaError_t make_intermediate_map(CUtensorMap* map, void* base, int ny, int px, int cap, int rows, int window = 0);
 cudaError_t launch_col(int py, const float2* win, long long win_item_stride, float2* wout,
                        long long wout_item_stride, int px, int items, const float4* tw,
                        const HParams& hp, cudaStream_t st);

@@ -1145,6 +1145,67 @@ cwo_status cwo_propagate(cwo_plan* plan, const void* in_c64, void* out_c64, void
     return run(plan, in_c64, (long long)plan->nx * plan->ny, out_c64, 1, nullptr, cuda_stream, false);
 }
 
+// rows are taken in groups of this many: a multiple of every row pass's group
+static constexpr int kRowGroup = 8;
+static bool rows_supported(const cwo_plan* p) {
+    return p->type == CWO_ANGULAR && !(p->hcache && p->py == cwo::kSplitColP);
+}
+
+}  // extern "C"
+
+bool cwo::plan_size(const cwo_plan* plan, int* nx, int* ny) {
+    if (!plan) return false;
+    *nx = plan->nx;
+    *ny = plan->ny;
+    return true;
+}
+
+extern "C" {
+
+int cwo_propagate_rows_group(const cwo_plan* plan) { return plan && rows_supported(plan) ? kRowGroup : 0; }
+
+cwo_status cwo_propagate_rows(cwo_plan* p, const void* in_c64, void* out_c64, int in_lo, int in_hi, int out_lo, int out_hi,
+                              int adjoint, void* cuda_stream) {
+    if (!p) return fail(CWO_ERR_INVALID_ARG, "plan is NULL");
+    if (!rows_supported(p)) return fail(CWO_ERR_UNSUPPORTED, "row windows are not provided for this plan");
+    if (in_lo < 0 || in_hi > p->ny || in_lo >= in_hi || out_lo < 0 || out_hi > p->ny || out_lo >= out_hi)
+        return fail(CWO_ERR_INVALID_ARG, "row windows must be non-empty and lie in [0, %d)", p->ny);
+    cwo_status st = check_plan_device(p);
+    if (st) return st;
+    const size_t fb = (size_t)p->nx * p->ny * sizeof(float2);
+    if ((st = check_device_range(in_c64, fb, p->device, "input")) || (st = check_device_range(out_c64, fb, p->device, "output")))
+        return st;
+    auto down = [](int y) { return y / kRowGroup * kRowGroup; };
+    auto up = [](int y) { return (y + kRowGroup - 1) / kRowGroup * kRowGroup; };
+    cwo::HParams hp = base_hparams(p, nullptr, 1);
+    hp.conj = adjoint ? 1 : 0;
+    if (p->hcache) {
+        hp.mode = cwo::HMODE_TABLE;
+        hp.hcache = p->hcache;
+        hp.hcache_stride = p->py;
+    }
+    hp.win = 1;
+    hp.ylo = down(in_lo); hp.yhi = up(in_hi);     // ny is a multiple of 16: up stays inside
+    hp.olo = down(out_lo); hp.ohi = up(out_hi);
+    // the row passes see the windows as fields of their own: the first row's address, the number of
+    // rows, and a tensor map of those rows of the intermediate
+    CUtensorMap mf, mi;
+    cudaError_t e;
+    if ((e = cwo::make_intermediate_map(&mf, p->scratch + hp.ylo, p->ny, p->px, 1, cwo::row_block_rows(p->px, false), hp.yhi - hp.ylo)) ||
+        (e = cwo::make_intermediate_map(&mi, p->scratch + hp.olo, p->ny, p->px, 1, cwo::row_block_rows(p->px, true), hp.ohi - hp.olo)))
+        return cuda_fail(e, "tensor map of a row window");
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    const long long field = (long long)p->nx * p->ny, wstride = (long long)p->ny * p->px;
+    const float scale = (float)(1.0 / ((double)p->px * (double)p->py));
+    if ((e = cwo::launch_row_fwd(p->px, (const float2*)in_c64 + (size_t)hp.ylo * p->nx, field, &mf, 0, hp.yhi - hp.ylo, 1, p->tw_x, p->status, s)))
+        return cuda_fail(e, "row forward launch");
+    if ((e = cwo::launch_col(p->py, p->scratch, wstride, p->scratch, wstride, p->px, 1, p->tw_y, hp, s)))
+        return cuda_fail(e, "column launch");
+    if ((e = cwo::launch_row_inv(p->px, &mi, 0, (float2*)out_c64 + (size_t)hp.olo * p->nx, field, hp.ohi - hp.olo, 1, scale, p->tw_x, p->status, s)))
+        return cuda_fail(e, "row inverse launch");
+    return CWO_OK;
+}
+
 cwo_status cwo_propagate_batch(cwo_plan* plan, const void* in, long long in_batch_stride, void* out,
                                int batch, const double* z_or_null, void* cuda_stream) {
     return run(plan, in, in_batch_stride, out, batch, z_or_null, cuda_stream, false);

@@ -26,11 +26,11 @@ static PFN_tensorMapEncodeTiled encode_fn() {
     return fn;
 }
 
-cudaError_t make_intermediate_map(CUtensorMap* map, void* base, int ny, int px, int cap, int rows) {
+cudaError_t make_intermediate_map(CUtensorMap* map, void* base, int ny, int px, int cap, int rows, int window) {
     PFN_tensorMapEncodeTiled fn = encode_fn();
     const int R = rows;
-    if (!fn || R < 2 || cap < 1 || ny % R) return cudaErrorInvalidValue;
-    const cuuint64_t dims[3] = {(cuuint64_t)ny, (cuuint64_t)px, (cuuint64_t)cap};
+    if (!fn || R < 2 || cap < 1 || ny % R || window % R || window > ny || (window && cap != 1)) return cudaErrorInvalidValue;
+    const cuuint64_t dims[3] = {(cuuint64_t)(window ? window : ny), (cuuint64_t)px, (cuuint64_t)cap};
     const cuuint64_t strides[2] = {(cuuint64_t)ny * sizeof(float2), (cuuint64_t)ny * px * sizeof(float2)};
     const cuuint32_t box[3] = {(cuuint32_t)R, (cuuint32_t)(px < kTmaBoxCols ? px : kTmaBoxCols), 1};
     const cuuint32_t estr[3] = {1, 1, 1};

@@ -114,11 +114,10 @@ def lib() -> ctypes.CDLL:
                 "cwo_launches_per_call": ([vp], i),
                 "cwo_propagate_epilogue": ([vp, vp, vp, i, i, i, vp, vp, vp], i),
                 "cwo_gs_run": ([vp, vp, vp, vp, i, i, vp], i),
-                "cwo_hologram_field": ([vp, i, i, i, i, i, i, vp, vp], i),
-                "cwo_hologram_intensity": ([vp, i, i, i, i, i, i, vp, vp], i),
-                "cwo_hologram_loss": ([vp, vp, i, i, i, i, i, i, vp, vp, vp, vp], i),
-                "cwo_hologram_seed": ([vp, vp, vp, i, i, i, i, i, i, vp, vp], i),
-                "cwo_hologram_phase_grad": ([vp, vp, i, i, i, i, i, i, vp, vp], i),
+                "cwo_hologram_forward": ([vp, vp, vp, i, i, i, i, vp, vp, vp, vp, vp], i),
+                "cwo_hologram_backward": ([vp, vp, vp, vp, vp, i, i, i, i, vp, vp, vp], i),
+                "cwo_propagate_rows": ([vp, vp, vp, i, i, i, i, i, vp], i),
+                "cwo_propagate_rows_group": ([vp], i),
                 "cwo_plan_check": ([vp], i),
                 "cwo_plan_set_timing_events": ([vp, ctypes.POINTER(ctypes.c_void_p)], i),
                 "cwo_last_error": ([], ctypes.c_char_p),
@@ -318,6 +317,24 @@ class Plan:
 
     def adjoint(self, x, out=None, stream=None):
         return self._one(lib().cwo_propagate_adjoint, "cwo_propagate_adjoint", x, out, stream)
+
+    @property
+    def rows_group(self) -> int:
+        """Rows per group of propagate_rows (0: this plan does not provide it)."""
+        return int(lib().cwo_propagate_rows_group(self.handle))
+
+    def propagate_rows(self, x, in_rows, out_rows, out=None, stream=None, adjoint=False):
+        """One field of which only the rows in_rows = (lo, hi) can be non-zero; of the result only the
+        rows out_rows are wanted.  Both are widened to whole groups of ``rows_group`` rows: input rows
+        of a touched group must hold their values (zeros outside the window), the other rows are not
+        read, and output rows of untouched groups are not written."""
+        _check_field(x, self.nx, self.ny, "input", 1)
+        out = self._result(x, out, x.shape[:-2], 1)
+        st = lib().cwo_propagate_rows(self.handle, x.data_ptr(), out.data_ptr(), int(in_rows[0]), int(in_rows[1]),
+                                      int(out_rows[0]), int(out_rows[1]), int(bool(adjoint)), _stream_handle(stream))
+        if st != OK:
+            check(st, "cwo_propagate_rows")
+        return out
 
     def propagate_batch(self, x, z=None, out=None, stream=None, adjoint=False):
         """Batch [B][Ny][Nx] -> [B][Ny][Nx].  ``z``: None (plan z) or B distances (host floats)."""

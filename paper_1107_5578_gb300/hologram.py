@@ -23,46 +23,51 @@ from . import autograd, cwo, synth
 
 class _Geometry:
     """The window of a problem on its canvas and the plan that propagates it, as they were at the call."""
-    __slots__ = ("plan", "args", "canvas")
+    __slots__ = ("plan", "window", "canvas")
 
     def __init__(self, p: "HologramProblem"):
         self.plan, self.canvas = p.plan, p.canvas
-        self.args = (p.h, p.w, p.canvas, p.canvas, p.ox, p.oy)
+        self.window = (p.h, p.w, p.ox, p.oy)
 
-    def propagated(self, phi):
-        """U = A exp(i phi) on the canvas"""
+    def forward(self, phi, target):
+        """(u, |u|^2) of u = A exp(i phi), or, with a target, (u, residual, loss)"""
         phi = phi.contiguous()
-        x = torch.empty(self.canvas, self.canvas, dtype=torch.complex64, device=phi.device)
-        _call("cwo_hologram_field", phi, *self.args, x)
-        return self.plan.propagate(x, out=x)
+        u = torch.empty(self.canvas, self.canvas, dtype=torch.complex64, device=phi.device)
+        image = torch.empty(phi.shape, dtype=torch.float32, device=phi.device)
+        if target is None:
+            _call("cwo_hologram_forward", self.plan.handle, phi.data_ptr(), None, *self.window, u.data_ptr(), image.data_ptr(), None, None)
+            return u, image
+        loss = torch.empty((), dtype=torch.float32, device=phi.device)
+        partial = torch.empty(cwo.HOLOGRAM_PARTIALS, dtype=torch.float64, device=phi.device)
+        _call("cwo_hologram_forward", self.plan.handle, phi.data_ptr(), target.data_ptr(), *self.window, u.data_ptr(), image.data_ptr(),
+              loss.data_ptr(), partial.data_ptr())
+        return u, image, loss
 
-    def phase_gradient(self, phi, u, gw, gl):
-        """A^H of the seed (through the adjoint kernels), and its derivative by the phase"""
-        phi, u, gw = phi.contiguous(), u.contiguous(), gw.contiguous()
-        g = torch.empty_like(u)
-        _call("cwo_hologram_seed", u, gw, gl, *self.args, g)
-        self.plan.adjoint(g, out=g)
-        out = torch.empty_like(phi)
-        _call("cwo_hologram_phase_grad", g, phi, *self.args, out)
+    def backward(self, phi, u, g, gloss):
+        """derivative by the phase, through the adjoint kernels"""
+        phi, u, g = phi.contiguous(), u.contiguous(), g.contiguous()
+        work, out = torch.empty_like(u), torch.empty_like(phi)
+        _call("cwo_hologram_backward", self.plan.handle, phi.data_ptr(), u.data_ptr(), g.data_ptr(),
+              None if gloss is None else gloss.data_ptr(), *self.window, work.data_ptr(), out.data_ptr())
         return out
 
     # the same steps as tensor operators: for inputs the kernels do not take, and for gradients of
     # gradients
     def field(self, phi):
-        h, w, _, _, ox, oy = self.args
+        h, w, ox, oy = self.window
         x = torch.zeros(self.canvas, self.canvas, dtype=torch.complex64, device=phi.device)
         x[oy:oy + h, ox:ox + w] = torch.polar(torch.ones_like(phi), phi)
         return x
 
     def intensity(self, phi):
-        h, w, _, _, ox, oy = self.args
+        h, w, ox, oy = self.window
         u = autograd.propagate(self.field(phi), self.plan)
         uw = u[oy:oy + h, ox:ox + w]
         return uw.real ** 2 + uw.imag ** 2
 
 
 def _call(name, *args):
-    st = getattr(cwo.lib(), name)(*(a.data_ptr() if isinstance(a, torch.Tensor) else a for a in args), cwo._stream_handle(None))
+    st = getattr(cwo.lib(), name)(*args, cwo._stream_handle(None))
     if st != cwo.OK:
         cwo.check(st, name)
 
@@ -72,19 +77,17 @@ class _Intensity(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, phi, geo):
-        u = geo.propagated(phi)
-        out = torch.empty(phi.shape, dtype=torch.float32, device=phi.device)
-        _call("cwo_hologram_intensity", u, *geo.args, out)
+        u, image = geo.forward(phi, None)
         ctx.geo = geo
         ctx.save_for_backward(phi, u)
-        return out
+        return image
 
     @staticmethod
     def backward(ctx, gi):
         phi, u = ctx.saved_tensors
         if torch.is_grad_enabled():   # a graph of the gradient is wanted: the composed operators have one
             return torch.autograd.grad(ctx.geo.intensity(phi), phi, gi, create_graph=True)[0], None
-        return ctx.geo.phase_gradient(phi, u, gi.resolve_neg(), None), None
+        return ctx.geo.backward(phi, u, gi.resolve_neg(), None), None
 
 
 class _Loss(torch.autograd.Function):
@@ -93,11 +96,7 @@ class _Loss(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, phi, target, geo):
-        u = geo.propagated(phi)
-        residual = torch.empty(phi.shape, dtype=torch.float32, device=phi.device)
-        loss = torch.empty((), dtype=torch.float32, device=phi.device)
-        partial = torch.empty(cwo.HOLOGRAM_PARTIALS, dtype=torch.float64, device=phi.device)
-        _call("cwo_hologram_loss", u, target, *geo.args, residual, loss, partial)
+        u, residual, loss = geo.forward(phi, target)
         ctx.geo = geo
         ctx.save_for_backward(phi, u, residual)
         return loss
@@ -109,7 +108,7 @@ class _Loss(torch.autograd.Function):
             inten = ctx.geo.intensity(phi)
             d = inten - (inten.detach() - residual)
             return torch.autograd.grad((d * d).mean(), phi, gl, create_graph=True)[0], None, None
-        return ctx.geo.phase_gradient(phi, u, residual, gl.resolve_neg()), None, None
+        return ctx.geo.backward(phi, u, residual, gl.resolve_neg()), None, None
 
 
 class HologramProblem:
@@ -119,7 +118,9 @@ class HologramProblem:
         self.oy, self.ox = (canvas - h) // 2, (canvas - w) // 2
         self.pitch, self.wavelength, self.z = pitch, wavelength, z
         self.device = torch.device(device)
-        self.plan = cwo.Plan(canvas, canvas, pitch, pitch, wavelength, z, cwo.ANGULAR)
+        # every propagation of the optimisation has the same distance: the transfer function is kept (67
+        # MB at 2048^2), except where the plan could then not propagate windows of rows
+        self.plan = cwo.Plan(canvas, canvas, pitch, pitch, wavelength, z, cwo.ANGULAR, cwo.FLAG_CACHE_H if canvas < 4096 else 0)
         phi0, tgt = synth.hologram_problem(seed, h, w)
         self.phi0 = phi0
         # scale the target so that its energy matches the initial field's intensity on the window

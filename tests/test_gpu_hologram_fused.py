@@ -70,9 +70,20 @@ def test_inputs_the_kernels_do_not_take(mods):
     p32 = phi.detach().float().requires_grad_(True)
     prob.loss(p32).backward()
     assert _rel(p32.grad, phi.grad) <= TOL
-    lib = __import__("paper_1107_5578_gb300.cwo", fromlist=["lib"])
+    from paper_1107_5578_gb300 import cwo
     x = torch.zeros(64, 64, dtype=torch.complex64, device="cuda")
+    image = torch.zeros(20, 30, device="cuda")
+    call = cwo.lib().cwo_hologram_forward
     for h, w, ox, oy in ((0, 5, 0, 0), (5, 5, 60, 0), (5, 5, 0, -1), (65, 5, 0, 0)):   # not inside the canvas
-        assert lib.lib().cwo_hologram_field(p32.data_ptr(), h, w, 64, 64, ox, oy, x.data_ptr(), 0) == lib.ERR_INVALID_ARG
+        assert call(prob.plan.handle, p32.data_ptr(), None, h, w, ox, oy, x.data_ptr(), image.data_ptr(), None, None, 0) \
+            == cwo.ERR_INVALID_ARG
     short = torch.zeros(16, device="cuda")
-    assert lib.lib().cwo_hologram_intensity(x.data_ptr(), 20, 30, 4096, 4096, 0, 0, short.data_ptr(), 0) == lib.ERR_INVALID_ARG
+    big = cwo.Plan(2048, 2048)
+    assert call(big.handle, p32.data_ptr(), None, 20, 30, 0, 0, short.data_ptr(), image.data_ptr(), None, None, 0) == cwo.ERR_INVALID_ARG
+    # a plan without row windows (a Fresnel one) propagates the whole canvas
+    prob.plan = cwo.Plan(64, 64, 6.4e-6, 6.4e-6, 520e-9, 0.01, cwo.FRESNEL_CONV)
+    assert prob.plan.rows_group == 0
+    geo = hologram._Geometry(prob)
+    (grad,) = torch.autograd.grad(prob.loss(p32), p32)
+    (want,) = torch.autograd.grad(want_loss(geo, prob, p32), p32)
+    assert _rel(grad, want) <= TOL
