@@ -67,9 +67,9 @@ k_col(const float2* __restrict__ win, long long win_item_stride, float2* __restr
 #pragma unroll
     for (int e = 8; e < 16; ++e) v[e] = make_float2(0.f, 0.f);   // zero padding rows
     const TwTable<P> twt{tw, t};
-    fwd1_from<P, C, 0, 8, false>(v, sm, c, t, twt);
+    fwd1_from<P, C, 0, 8, false, P == 4096>(v, sm, c, t, twt);
     apply_h<P, 1, MIXED>(v, v, col, t, item, hp);
-    inv1_from<P, C, Geo<P>::NST - 1, false>(v, sm, c, t, twt);
+    inv1_from<P, C, Geo<P>::NST - 1, false, P == 4096>(v, sm, c, t, twt);
     float2* dst = wout + item * wout_item_stride + (long long)col * NY;
 #pragma unroll
     for (int e = 0; e < 8; ++e) dst[t + e * T] = v[e];           // crop: rows < Ny
@@ -153,9 +153,10 @@ k_colp(const float2* __restrict__ win, long long win_item_stride, float2* __rest
 #pragma unroll
     for (int e = 8; e < 16; ++e) { a[e] = make_float2(0.f, 0.f); b[e] = make_float2(0.f, 0.f); }
     if constexpr (P >= 128) {
-        fwd2v_from<P, CP, 0, 8>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
+        constexpr bool MERGED = P == 4096;
+        fwd2v_from<P, CP, 0, 8, MERGED>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
         apply_h<P, 2, MIXED>(a, b, pr.x, t, item, hp);
-        inv2v_from<P, CP, Geo<P>::NST - 1>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
+        inv2v_from<P, CP, Geo<P>::NST - 1, MERGED>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
     } else {
         using Lay = PadLayout<P, 2 * CP>;
         fwd2x_from<P, CP, Lay, 0, 8>(a, b, sm, cp, t, tw);

@@ -42,25 +42,26 @@ void emu_exchange(std::vector<Regs>& R) {
         for (int e = 0; e < 16; ++e) R[t].v[e] = sm[PadLayout<P, 1>::addr(0, stage_pos<P, SR>(t, e))];
 }
 
-template <int P, int S, int NZ0>
+// MERGED as in the kernels: the plain columns and lines of P = 4096 (not the split column pass)
+template <int P, int S, int NZ0, bool MERGED = P == 4096>
 void emu_fwd_from(std::vector<Regs>& R, const float4* tw) {
     using G = Geo<P>;
-    for (int t = 0; t < G::T; ++t) stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16)>(R[t].v);
+    for (int t = 0; t < G::T; ++t) stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16), MERGED>(R[t].v);
     if constexpr (S < G::NST - 1) {
         emu_twiddle<P, S, false>(R, tw);
         emu_exchange<P, S, S + 1>(R);
-        emu_fwd_from<P, S + 1, NZ0>(R, tw);
+        emu_fwd_from<P, S + 1, NZ0, MERGED>(R, tw);
     }
 }
 
-template <int P, int S>
+template <int P, int S, bool MERGED = P == 4096>
 void emu_inv_from(std::vector<Regs>& R, const float4* tw) {
     using G = Geo<P>;
     if constexpr (S < G::NST - 1) emu_twiddle<P, S, true>(R, tw);
-    for (int t = 0; t < G::T; ++t) stage_butterflies<P, S, true, 16>(R[t].v);
+    for (int t = 0; t < G::T; ++t) stage_butterflies<P, S, true, 16, MERGED>(R[t].v);
     if constexpr (S > 0) {
         emu_exchange<P, S, S - 1>(R);
-        emu_inv_from<P, S - 1>(R, tw);
+        emu_inv_from<P, S - 1, MERGED>(R, tw);
     }
 }
 
@@ -102,16 +103,16 @@ void emu_col_split(float2* col, long long step, const float2* w, const float4* t
             A[t].v[e] = col[(long long)(t + e * T) * step];
             B[t].v[e] = cmul(A[t].v[e], w[t + e * T]);
         }
-    emu_fwd_from<Q, 0, 16>(A, twq);
-    emu_fwd_from<Q, 0, 16>(B, twq);
+    emu_fwd_from<Q, 0, 16, false>(A, twq);
+    emu_fwd_from<Q, 0, 16, false>(B, twq);
     for (int t = 0; t < T; ++t)
         for (int e = 0; e < 16; ++e) {
             const float2 ha = hs[e * T + t], hb = hs[Q + e * T + t];
             A[t].v[e] = adjoint ? cmulc(A[t].v[e], ha) : cmul(A[t].v[e], ha);
             B[t].v[e] = adjoint ? cmulc(B[t].v[e], hb) : cmul(B[t].v[e], hb);
         }
-    emu_inv_from<Q, Geo<Q>::NST - 1>(A, twq);
-    emu_inv_from<Q, Geo<Q>::NST - 1>(B, twq);
+    emu_inv_from<Q, Geo<Q>::NST - 1, false>(A, twq);
+    emu_inv_from<Q, Geo<Q>::NST - 1, false>(B, twq);
     for (int t = 0; t < T; ++t)
         for (int e = 0; e < 16; ++e)
             col[(long long)(t + e * T) * step] = cadd(A[t].v[e], cmulc(B[t].v[e], w[t + e * T]));

@@ -157,11 +157,84 @@ CWO_HD void dft16(float2 (&v)[16]) {
         for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = w[4 * k1 + k2];
 }
 
+// The same 16-point DFT as radix-2 levels whose roots of unity are merged into the sums: with w = c (1 +
+// i t) the butterfly a +- w b takes two multiply-adds for b (1 + i t) and four for the sums (Linzer and
+// Feig, "Implementation of efficient FFT algorithms on fused multiply-add architectures", 1993), c and t
+// immediates.  148 instructions instead of 160 and one rounding less per merged root; alone, with two
+// transforms a thread and four warps a scheduler, 613 against 677 ns a stage.  (With twiddles from
+// memory in that form a stage took 1077 against 961 ns, although 384 against 440 instructions: a
+// multiply-add of three registers issues at 0.73 a cycle.)  In a whole kernel registers and the order
+// of the instructions decide: it is used where it measured faster, at P = 4096 in the pair kernels
+// (column pass of 16 2048^2 fields 934 -> 914 us, Fresnel line passes 1076 -> 1047), the inverse row pass
+// (361 -> 355), the stack's first pass (342 -> 334) and the single-column kernel (4 fields 294 -> 283), and
+// not in the forward row pass there (357 -> 359), at P <= 2048 (0 to 3% slower) or in the split column
+// pass (598 -> 616).
+CWO_HD void bf(float2& a, float2& b) {
+    const float2 u = cadd(a, b);
+    b = csub(a, b);
+    a = u;
+}
+template <bool INV> CWO_HD void bf_w4(float2& a, float2& b) {
+    const float2 r = mul_w4<INV>(b);
+    b = csub(a, r);
+    a = cadd(a, r);
+}
+// w = W_16^E, E = 1, 2, 3; W4: times W_4
+template <bool INV, int E, bool W4> CWO_HD void bf_root(float2& a, float2& b) {
+    constexpr float c = E == 1 ? kCos1 : E == 2 ? kRsqrt2 : kSin1;
+    constexpr float t = (INV ? 1.0f : -1.0f) * (E == 1 ? 0.41421356237309504880f : E == 2 ? 1.0f : 2.41421356237309504880f);
+    const float p = fmaf(-t, b.y, b.x), q = fmaf(t, b.x, b.y);
+    if constexpr (W4) {
+        constexpr float s = INV ? -c : c;
+        b = make_float2(fmaf(-s, q, a.x), fmaf(s, p, a.y));
+        a = make_float2(fmaf(s, q, a.x), fmaf(-s, p, a.y));
+    } else {
+        b = make_float2(fmaf(-c, p, a.x), fmaf(-c, q, a.y));
+        a = make_float2(fmaf(c, p, a.x), fmaf(c, q, a.y));
+    }
+}
+template <bool INV, int NZ>
+CWO_HD void dft16_merged(float2 (&v)[16]) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        if constexpr (NZ == 8) v[e + 8] = v[e];
+        else bf(v[e], v[e + 8]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        bf(v[e], v[e + 4]);
+        bf_w4<INV>(v[e + 8], v[e + 12]);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        bf(v[e], v[e + 2]);
+        bf_w4<INV>(v[e + 4], v[e + 6]);
+        bf_root<INV, 2, false>(v[e + 8], v[e + 10]);
+        bf_root<INV, 2, true>(v[e + 12], v[e + 14]);
+    }
+    bf(v[0], v[1]);
+    bf_w4<INV>(v[2], v[3]);
+    bf_root<INV, 2, false>(v[4], v[5]);
+    bf_root<INV, 2, true>(v[6], v[7]);
+    bf_root<INV, 1, false>(v[8], v[9]);
+    bf_root<INV, 1, true>(v[10], v[11]);
+    bf_root<INV, 3, false>(v[12], v[13]);
+    bf_root<INV, 3, true>(v[14], v[15]);
+    // the levels leave the outputs in bit-reversed order
+    float2 w[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i] = v[i];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[((i & 1) << 3) | ((i & 2) << 1) | ((i & 4) >> 1) | ((i & 8) >> 3)] = w[i];
+}
+
 // the butterflies of stage S on a thread's 16 registers
-template <int P, int S, bool INV, int NZ>
+template <int P, int S, bool INV, int NZ, bool MERGED = false>
 CWO_HD void stage_butterflies(float2 (&v)[16]) {
     constexpr int R = Geo<P>::radix(S);
-    if constexpr (R == 16) {
+    if constexpr (R == 16 && MERGED) {
+        dft16_merged<INV, NZ>(v);
+    } else if constexpr (R == 16) {
         dft16<INV, NZ>(v);
     } else if constexpr (R == 8) {
         dft8<INV, 0>(v); dft8<INV, 8>(v);
@@ -297,32 +370,32 @@ __device__ __forceinline__ void xch1(float2* __restrict__ sm, int r, int t, floa
 
 // forward DIF from stage S to the end / adjoint from stage S down to stage 0 (or, for
 // inv1_to_stage0, down to and including the exchange into stage 0), with xch1 exchanges
-template <int P, int R, int S, int NZ0, bool IL = true, class Tw>
+template <int P, int R, int S, int NZ0, bool IL = true, bool MERGED = false, class Tw>
 __device__ __forceinline__ void fwd1_from(float2 (&v)[16], float2* __restrict__ sm, int r, int t, const Tw& tw) {
-    stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16)>(v);
+    stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16), MERGED>(v);
     if constexpr (S < Geo<P>::NST - 1) {
         tw.template apply<S, false>(v);
         xch1<P, R, S, S + 1, IL>(sm, r, t, v);
-        fwd1_from<P, R, S + 1, NZ0, IL>(v, sm, r, t, tw);
+        fwd1_from<P, R, S + 1, NZ0, IL, MERGED>(v, sm, r, t, tw);
     }
 }
 
-template <int P, int R, int S, bool IL = true, class Tw>
+template <int P, int R, int S, bool IL = true, bool MERGED = false, class Tw>
 __device__ __forceinline__ void inv1_from(float2 (&v)[16], float2* __restrict__ sm, int r, int t, const Tw& tw) {
     if constexpr (S < Geo<P>::NST - 1) tw.template apply<S, true>(v);
-    stage_butterflies<P, S, true, 16>(v);
+    stage_butterflies<P, S, true, 16, MERGED>(v);
     if constexpr (S > 0) {
         xch1<P, R, S, S - 1, IL>(sm, r, t, v);
-        inv1_from<P, R, S - 1, IL>(v, sm, r, t, tw);
+        inv1_from<P, R, S - 1, IL, MERGED>(v, sm, r, t, tw);
     }
 }
 
-template <int P, int R, int S, class Tw>
+template <int P, int R, int S, bool MERGED = false, class Tw>
 __device__ __forceinline__ void inv1_to_stage0(float2 (&v)[16], float2* __restrict__ sm, int r, int t, const Tw& tw) {
     if constexpr (S < Geo<P>::NST - 1) tw.template apply<S, true>(v);
-    stage_butterflies<P, S, true, 16>(v);
+    stage_butterflies<P, S, true, 16, MERGED>(v);
     xch1<P, R, S, S - 1>(sm, r, t, v);
-    if constexpr (S > 1) inv1_to_stage0<P, R, S - 1>(v, sm, r, t, tw);
+    if constexpr (S > 1) inv1_to_stage0<P, R, S - 1, MERGED>(v, sm, r, t, tw);
 }
 
 template <int P, int CP, class Lay, int SW, int SR>
@@ -365,30 +438,31 @@ __device__ __forceinline__ void xch2v(float4* __restrict__ sm, int cp, int t, fl
     }
 }
 
-// forward / inverse stages of a pair with the 128-bit exchange (P >= 128)
-template <int P, int CP, int S, int NZ0>
+// forward / inverse stages of a pair with the 128-bit exchange (P >= 128); MERGED: the 16-point DFTs with
+// merged roots
+template <int P, int CP, int S, int NZ0, bool MERGED = false>
 __device__ __forceinline__ void fwd2v_from(float2 (&a)[16], float2 (&b)[16], float4* __restrict__ sm, int cp, int t,
                                            const float4* __restrict__ tw) {
     using G = Geo<P>;
-    stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16)>(a);
-    stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16)>(b);
+    stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16), MERGED>(a);
+    stage_butterflies<P, S, false, (S == 0 ? NZ0 : 16), MERGED>(b);
     if constexpr (S < G::NST - 1) {
         twiddle2<P, S, false>(a, b, tw, t);
         xch2v<P, CP, S, S + 1>(sm, cp, t, a, b);
-        fwd2v_from<P, CP, S + 1, NZ0>(a, b, sm, cp, t, tw);
+        fwd2v_from<P, CP, S + 1, NZ0, MERGED>(a, b, sm, cp, t, tw);
     }
 }
 
-template <int P, int CP, int S>
+template <int P, int CP, int S, bool MERGED = false>
 __device__ __forceinline__ void inv2v_from(float2 (&a)[16], float2 (&b)[16], float4* __restrict__ sm, int cp, int t,
                                            const float4* __restrict__ tw) {
     using G = Geo<P>;
     if constexpr (S < G::NST - 1) twiddle2<P, S, true>(a, b, tw, t);
-    stage_butterflies<P, S, true, 16>(a);
-    stage_butterflies<P, S, true, 16>(b);
+    stage_butterflies<P, S, true, 16, MERGED>(a);
+    stage_butterflies<P, S, true, 16, MERGED>(b);
     if constexpr (S > 0) {
         xch2v<P, CP, S, S - 1>(sm, cp, t, a, b);
-        inv2v_from<P, CP, S - 1>(a, b, sm, cp, t, tw);
+        inv2v_from<P, CP, S - 1, MERGED>(a, b, sm, cp, t, tw);
     }
 }
 

@@ -310,9 +310,10 @@ k_line_pair(const float2* __restrict__ in, long long in_item_stride, const __gri
             b[e] = conj ? cmulc(b[e], w) : cmul(b[e], w);
         }
     };
-    fwd2v_from<P, CP, 0, 8>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
+    constexpr bool MERGED = P == 4096;
+    fwd2v_from<P, CP, 0, 8, MERGED>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
     mul_h();
-    inv2v_from<P, CP, Geo<P>::NST - 1>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
+    inv2v_from<P, CP, Geo<P>::NST - 1, MERGED>(a, b, reinterpret_cast<float4*>(sm), cp, t, tw);
     constexpr int R = 2 * CP, BOX = N < kTmaBoxCols ? N : kTmaBoxCols;
     __syncthreads();   // every exchange read done before the tile (which aliases the region) is written
 #pragma unroll
@@ -393,7 +394,7 @@ k_line_stack_p(const float2* __restrict__ in, const __grid_constant__ CUtensorMa
         fence_proxy_async_smem();   // these reads of the staging buffer precede the next bulk copy into it
         if (__syncthreads_or(!ok)) break;                                // a copy did not land
         if (threadIdx.x == 0 && g + (int)gridDim.x < groups) issue(g + gridDim.x);
-        fwd1_from<P, R, 0, 8>(spec, sm, r, t, twt);
+        fwd1_from<P, R, 0, 8, true, P == 4096>(spec, sm, r, t, twt);
 #pragma unroll 1
         for (int j = 0; j < planes; ++j, ++np) {
             float2* tile = tiles + (np & 1) * R * N;
@@ -406,7 +407,7 @@ k_line_stack_p(const float2* __restrict__ in, const __grid_constant__ CUtensorMa
                 const float2 w = __ldg(hh + e * T);
                 v[e] = conj ? cmulc(spec[e], w) : cmul(spec[e], w);
             }
-            inv1_from<P, R, Geo<P>::NST - 1>(v, sm, r, t, twt);
+            inv1_from<P, R, Geo<P>::NST - 1, true, P == 4096>(v, sm, r, t, twt);
 #pragma unroll
             for (int e = 0; e < 8; ++e) tile[e * NT + threadIdx.x] = cscale(v[e], scale);
             fence_proxy_async_smem();

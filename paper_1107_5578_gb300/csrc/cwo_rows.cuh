@@ -392,12 +392,12 @@ k_row_inv_p(const __grid_constant__ CUtensorMap wmap, int item_off, float2* __re
 #pragma unroll
         for (int e = 0; e < 16; ++e) v[e] = sm[e * NT + threadIdx.x];
         if (__syncthreads_or(!ok)) break;          // a copy did not land: the status word says so
-        inv1_to_stage0<P, R, Geo<P>::NST - 1>(v, sm, r, t, twt);
+        inv1_to_stage0<P, R, Geo<P>::NST - 1, P == 4096>(v, sm, r, t, twt);
         fence_proxy_async_smem();                  // the exchange reads precede the next tile load
         __syncthreads();
         if (threadIdx.x == 0 && g + (int)gridDim.x < total_groups) issue(g + gridDim.x);
         twt.template apply<0, true>(v);
-        stage_butterflies<P, 0, true, 16>(v);
+        stage_butterflies<P, 0, true, 16, P == 4096>(v);
         const int item = g / groups_per_item, y0 = (g % groups_per_item) * R;
         const long long base = item * out_item_stride + (long long)(y0 + r) * N;
 #pragma unroll
