@@ -31,21 +31,18 @@ def test_axis_of_4096(gpu, nx, ny, form):
     batch, z = 3, 0.03
     u = np.stack([synth.random_field(nx, seed=nx + ny + k, ny=ny) for k in range(batch)])
     x = torch.from_numpy(u.astype(np.complex64)).cuda()
-    kw, zs, want = {}, [z] * batch, lambda k: oracle.propagate(u[k], 8e-6, 8e-6, 532e-9, z, kw.get("kind", 0))
+    kind = cwo.FRESNEL_CONV if form in ("fresnel", "stack") else cwo.ANGULAR
+    kw, zs, want = {}, [z] * batch, lambda k: oracle.propagate(u[k], 8e-6, 8e-6, 532e-9, z, kind)
     if form == "cached":
         kw["flags"] = cwo.FLAG_CACHE_H
-    elif form in ("fresnel", "stack"):
-        kw["kind"] = cwo.FRESNEL_CONV
     elif form == "shifted":
         kw["shift"] = cwo.Shift(2e-4, -1e-4, 0.0, 0.0, 0.0, 0.0)
         want = lambda k: oracle.propagate_shifted(u[k], 8e-6, 8e-6, 532e-9, z, 2e-4, -1e-4, 0.0, 0.0, 0.0, 0.0)
     if form == "stack":
         zs = [0.03, 0.05, -0.04]
-        x = x[:1].expand(batch, ny, nx)
         want = lambda k: oracle.propagate(u[0], 8e-6, 8e-6, 532e-9, zs[k], cwo.FRESNEL_CONV)
-    kind = kw.pop("kind", cwo.ANGULAR)
     plan = cwo.Plan(nx, ny, 8e-6, 8e-6, 532e-9, z, kind, **kw)
-    y = plan.propagate_batch(x, **({"z": zs} if form == "stack" else {})).cpu().numpy()
+    y = (plan.propagate_stack(x[0].contiguous(), zs) if form == "stack" else plan.propagate_batch(x)).cpu().numpy()
     plan.check()
     plan.close()
     for k in range(batch):
