@@ -191,8 +191,8 @@ cwo_status cwo_propagate(cwo_plan* plan, const void* in_c64, void* out_c64, void
  *                    its spectrum is computed once and reused for every plane.
  *   out              [batch][Ny][Nx]
  *   z_or_null        NULL: every item uses the plan's z.  Otherwise a HOST array of `batch`
- *                    distances; the per-item tables are computed in FP64 on the host and uploaded
- *                    stream-ordered.
+ *                    distances; the per-item tables are computed in FP64, stream-ordered (angular
+ *                    spectrum: on the device; Fresnel: on the host and uploaded).
  * Grows the scratch (synchronising) if `batch` exceeds the reserved size.
  * Any complex64-aligned (8-byte) buffers are accepted; fields whose rows start on 16-byte
  * boundaries take the kernels that move them by bulk and TMA copies (the fastest paths), others
@@ -227,8 +227,8 @@ typedef struct {
  * distance, wavelength, pitches) -- the batching step of a serving loop that groups same-size
  * requests.  The plan supplies the shape, the scratch and the FFT tables; its own wavelength,
  * pitches, distance and type are not used.  items is a HOST array; the per-item
- * transfer-function tables are computed in FP64 on the host (in parallel threads) and uploaded
- * stream-ordered.  in_batch_stride as in cwo_propagate_batch but must be > 0.  Each contiguous
+ * transfer-function tables are computed in FP64, stream-ordered: angular spectrum on the device,
+ * Fresnel on the host (in parallel threads) and uploaded.  in_batch_stride as in cwo_propagate_batch but must be > 0.  Each contiguous
  * run of angular-spectrum items is one set of three launches; each contiguous run of Fresnel
  * items, the two separable line passes of a Fresnel plan (three launches instead when out is not
  * on a 16-byte boundary), so a caller that orders its batch by type makes at most five launches.
