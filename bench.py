@@ -123,17 +123,20 @@ class ClockSampler:
 
 
 # ---- FP32 arithmetic of the passes, counted from the kernels' own butterflies (P = 4096: three
-# radix-16 DIF stages).  FP32 instructions per 16 points: a radix-16 butterfly done as 4 x 4
-# (eight radix-4 DFTs of 16 additions, eight non-trivial inner twiddles of 4 instructions) = 160;
-# the first forward stage, whose upper 8 inputs are the zero padding, 128; the last inverse stage,
-# of which only the lower 8 outputs are kept, 144; the 15 inter-stage twiddle multiplications
-# (complex multiply = 2 FMUL + 2 FFMA) 60.  ncu counts of the same kernels (fadd + fmul + ffma
-# thread instructions) agree within 4% (profiles/asm_2048_kernels_full.md).
-FP32_R16, FP32_R16_ZERO_HALF_IN, FP32_R16_HALF_OUT, FP32_TWIDDLES = 160, 128, 144, 60
-FP32_FWD = (FP32_R16_ZERO_HALF_IN + FP32_TWIDDLES + FP32_R16 + FP32_TWIDDLES + FP32_R16) / 16.0   # per point
-FP32_INV = (FP32_R16 + FP32_TWIDDLES + FP32_R16 + FP32_TWIDDLES + FP32_R16_HALF_OUT) / 16.0       # per point
+# radix-16 DIF stages).  FP32 instructions per 16 points: the forward row pass's radix-16 butterfly,
+# done as 4 x 4 (eight radix-4 DFTs of 16 additions, eight non-trivial inner twiddles of 4
+# instructions) = 160, and 128 in the first stage, whose upper 8 inputs are the zero padding; the
+# other passes' butterfly with merged roots (22 radix-2 butterflies of 4 instructions, 10 of 6) = 148,
+# 116 with zero upper inputs and 132 in the last inverse stage, of which only the lower 8 outputs are
+# kept; the 15 inter-stage twiddle multiplications (complex multiply = 2 FMUL + 2 FFMA) 60.  ncu counts
+# of the same kernels (fadd + fmul + ffma thread instructions) agree within 4% for the forward row pass
+# and exactly for the others (profiles/asm_split_rows_and_merged_roots.md).
+FP32_TWIDDLES = 60
+FP32_ROW_FWD = (128 + FP32_TWIDDLES + 160 + FP32_TWIDDLES + 160) / 16.0   # per point
+FP32_FWD = (116 + FP32_TWIDDLES + 148 + FP32_TWIDDLES + 148) / 16.0
+FP32_INV = (148 + FP32_TWIDDLES + 148 + FP32_TWIDDLES + 132) / 16.0
 FP32_PER_PASS = {   # FP32 instructions per propagation of an N x N field (P = 2N)
-    "row_fwd": FP32_FWD * N * 2 * N,                      # N rows of P points
+    "row_fwd": FP32_ROW_FWD * N * 2 * N,                      # N rows of P points
     "col_fwd_h_inv": (FP32_FWD + 4.0 + FP32_INV) * (2 * N) ** 2,   # P columns: FFT, x H (loaded), IFFT
     "row_inv": (FP32_INV + 1.0) * N * 2 * N,              # N rows: IFFT, 1/(Px Py) on the kept half
 }
