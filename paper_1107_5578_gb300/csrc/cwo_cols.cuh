@@ -67,9 +67,10 @@ k_col(const float2* __restrict__ win, long long win_item_stride, float2* __restr
 #pragma unroll
     for (int e = 8; e < 16; ++e) v[e] = make_float2(0.f, 0.f);   // zero padding rows
     const TwTable<P> twt{tw, t};
-    fwd1_from<P, C, 0, 8, false, P == 4096>(v, sm, c, t, twt);
+    constexpr bool MERGED = P == 4096 || P == 2048;   // where it measured faster
+    fwd1_from<P, C, 0, 8, false, MERGED>(v, sm, c, t, twt);
     apply_h<P, 1, MIXED>(v, v, col, t, item, hp);
-    inv1_from<P, C, Geo<P>::NST - 1, false, P == 4096>(v, sm, c, t, twt);
+    inv1_from<P, C, Geo<P>::NST - 1, false, MERGED>(v, sm, c, t, twt);
     float2* dst = wout + item * wout_item_stride + (long long)col * NY;
 #pragma unroll
     for (int e = 0; e < 8; ++e) dst[t + e * T] = v[e];           // crop: rows < Ny

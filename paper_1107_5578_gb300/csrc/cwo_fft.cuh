@@ -166,9 +166,10 @@ CWO_HD void dft16(float2 (&v)[16]) {
 // multiply-add of three registers issues at 0.73 a cycle.)  In a whole kernel registers and the order
 // of the instructions decide: it is used where it measured faster, at P = 4096 in the pair kernels
 // (column pass of 16 2048^2 fields 934 -> 914 us, Fresnel line passes 1076 -> 1047), the inverse row pass
-// (361 -> 355), the stack's first pass (342 -> 334) and the single-column kernel (4 fields 294 -> 283), and
-// not in the forward row pass there (357 -> 359), at P <= 2048 (0 to 3% slower) or in the split column
-// pass (598 -> 616).
+// (361 -> 355), the stack's first pass (342 -> 334) and the single-column kernel (4 fields 294 -> 283; at
+// P = 2048, 3 fields of 4096 x 1024, 195.2 -> 193.1), and in the inverse split row pass (2 4096^2 fields 238.4
+// -> 236.0).  Not in the forward row pass (357 -> 359), elsewhere at P <= 2048 (0 to 3% slower), in the split
+// column pass (598 -> 616) or the 8192-point line pass (197.3 -> 199.7).
 CWO_HD void bf(float2& a, float2& b) {
     const float2 u = cadd(a, b);
     b = csub(a, b);

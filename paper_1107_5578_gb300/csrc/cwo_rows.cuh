@@ -332,12 +332,12 @@ k_row_inv_s(const __grid_constant__ CUtensorMap wmap, int item_off, float2* __re
             if (h == 0 || g + (int)gridDim.x < total_groups) mbar_wait_bounded(mbar + (h ^ 1), h == 0 ? parity : parity ^ 1u, status);
             break;
         }
-        inv1_to_stage0<Q, R, Geo<Q>::NST - 1>(v, buf, r, t, twt);
+        inv1_to_stage0<Q, R, Geo<Q>::NST - 1, true>(v, buf, r, t, twt);
         fence_proxy_async_smem();      // the exchange reads precede the next tile load
         __syncthreads();
         if (threadIdx.x == 0 && g + (int)gridDim.x < total_groups) issue(g + gridDim.x, h);
         twt.template apply<0, true>(v);
-        stage_butterflies<Q, 0, true, 16>(v);
+        stage_butterflies<Q, 0, true, 16, true>(v);
         if (h == 0) {
 #pragma unroll
             for (int e = 0; e < 16; ++e) even[e] = v[e];

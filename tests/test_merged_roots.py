@@ -1,4 +1,4 @@
-"""The 16-point DFT with merged roots (padded length 4096) against the oracle.  Bounds: a padded 4096-point
+"""The 16-point DFT with merged roots (padded length 4096; 2048 in shifted plans, 8192 in split rows) against the oracle.  Bounds: a padded 4096-point
 transform pair rounds each value about 2 x 12 levels at 6e-8, rms about 6e-8 sqrt(24) = 3e-7 an axis; with
 the tables' 1e-7 a value under 1e-6, and four times that is allowed."""
 import numpy as np
@@ -24,7 +24,7 @@ def test_emulated_axis_of_4096(nx, ny, kind, z, adjoint):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("nx,ny", [(16, 2048), (2048, 32), (512, 2048), (2048, 512)])
+@pytest.mark.parametrize("nx,ny", [(16, 2048), (2048, 32), (512, 2048), (2048, 512), (32, 1024), (4096, 1024)])
 @pytest.mark.parametrize("form", ["asm", "cached", "fresnel", "shifted", "stack"])
 def test_axis_of_4096(gpu, nx, ny, form):
     import torch
