@@ -6,7 +6,7 @@
 // upload of 16 bytes an entry; here each entry is one thread, and the parameters of up to
 // kAsmItems items travel in the launch: a batch of 12 512^2 items (4 of them Fresnel) took 132 us of
 // host time before.  The unit is compiled without contraction of multiplies and adds (as is
-// cwo_tables.cpp), so that the entries are the host's bit for bit.
+// cwo_asm_tables.cpp), so that the entries are the host's bit for bit.
 #include "cwo_internal.h"
 #include "cwo_launch.cuh"
 #include "cwo_tables.h"

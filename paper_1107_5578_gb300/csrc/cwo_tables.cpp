@@ -176,6 +176,11 @@ const AxisCache& axis_cache(int P, bool split = false) {
 }
 }  // namespace
 
+MirrorIndices mirror_indices(const AxisGeo& g) {
+    const AxisCache& c = axis_cache(g.P, g.split);
+    return {c.first.data(), c.second.data()};
+}
+
 // Forward DFT in FP64 (self-sorting Stockham form): one radix-2 pass when log2 n is odd, then
 // radix-4 passes.  A pass of radix r takes x[j m + k + q l' m] (q < r) to
 // y[(r j + q) m + k] = (sum_p x_p W_r^{p q}) W_n^{j q m}, with l' = l / r, for j < l', k < m.
@@ -294,17 +299,6 @@ AsmAxis asm_axis(int P, double pitch, double lambda, double z, bool is_x) {
     A.c0 = is_x ? frac01(K) : 0.0;
     A.su = (is_x && K < 0 ? -1.0 : 1.0) * (std::sqrt(std::fabs(K)) * 0.5);
     return A;
-}
-
-void asm_axis_table(const AxisGeo& g, double pitch, double lambda, double z, bool is_x, float4* out) {
-    const AsmAxis A = asm_axis(g.P, pitch, lambda, z, is_x);
-    // every entry depends on kt^2 only: evaluate |kt| = 0 .. P/2 once, store at both indices
-    const AxisCache& c = axis_cache(g.P, g.split);
-    for (int k = 0; k <= g.P / 2; ++k) {
-        const float4 v = asm_axis_entry(A, (double)k * (double)k);
-        out[c.first[k]] = v;
-        if (c.second[k] >= 0) out[c.second[k]] = v;
-    }
 }
 
 bool in_window(double f, double wc, double ww) { return !(ww > 0) || std::fabs(f - wc) <= 0.5 * ww; }

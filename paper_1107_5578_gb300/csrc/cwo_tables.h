@@ -36,6 +36,9 @@ const std::vector<float4>& twiddle_table(const AxisGeo& g);
 std::vector<int> bin_table(const AxisGeo& g);
 // storage columns of the frequencies +k and -k for k = 0 .. P/2 (0 and P/2 pair with themselves)
 std::vector<int2> mirror_pairs(const AxisGeo& g);
+// axis indices of the bins +k and -k for k = 0 .. P/2 (-1: the bin is its own mirror); kept as the tables are
+struct MirrorIndices { const int* first; const int* second; };
+MirrorIndices mirror_indices(const AxisGeo& g);
 // Split form of a zero-padded axis of P = 2Q points carrying Q samples x_n: its DFT is the pair of
 // Q-point DFTs of x_n (frequencies 2k) and of x_n W_P^n (frequencies 2k + 1).  Split axis index
 // i = h Q + idx (h = 0 even, 1 odd; idx a Q-point axis index) holds frequency 2 k(idx) + h.
