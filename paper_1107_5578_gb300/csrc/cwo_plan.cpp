@@ -115,13 +115,15 @@ cwo_status upload(T* dst, const std::vector<T>& src, const char* what) {
 // field and once: 64 512^2 fields 393 and 361, 24 149 and 146, 16 1024^2 403 and 388, 64 256^2 101 and
 // 96; but 4 1024^2 fields 112 and 116.  Sides up to kSharedHSide: larger tables (67 MB at 2048^2) are
 // left to CWO_FLAG_CACHE_H, whose user has asked for the memory.
+// The table (Nx + 1 columns of 2 Ny) lies in the scratch of the field after the batch's last (Nx such columns),
+// which cwo_plan_reserve holds for a stack's source; scratch_entries adds the last column.
 constexpr int kSharedHBatch = 8;
 constexpr size_t kSharedHValues = (size_t)1 << 24;
 constexpr int kSharedHSide = 1024;
-size_t shared_h_entries(int nx, int ny, int batch) {
-    const bool worth = batch >= kSharedHBatch && (size_t)batch * (2 * nx) * (2 * ny) >= kSharedHValues;
-    return worth && std::max(nx, ny) <= kSharedHSide ? (size_t)(nx + 1) * 2 * ny : 0;
+bool shared_h_worth(int nx, int ny, int batch) {
+    return batch >= kSharedHBatch && (size_t)batch * (2 * nx) * (2 * ny) >= kSharedHValues && std::max(nx, ny) <= kSharedHSide;
 }
+size_t scratch_entries(int ny, int px, int items) { return (size_t)items * ny * px + 2 * (size_t)ny; }
 
 size_t tables_bytes(int nx, int ny) {
     const AxisGeo gx(2 * nx), gy(2 * ny);
@@ -218,8 +220,6 @@ struct cwo_plan {
     cwo_shifted_fresnel sfr{};
     // CWO_FLAG_CACHE_H: the ASM transfer function of the plan's own z, [Px/2 + 1 pairs][Py]
     float2* hcache = nullptr;
-    // the same for one call of a batch (shared_h_entries; null: none, the fields evaluate H themselves)
-    float2* hshared = nullptr;
     // an axis of 8192 points in the split form (the row passes, and the column pass with a cached
     // transfer function): the 4096-point twiddles, then W_8192^n (float2).  Every table along x is then
     // in the split order, but for the Fresnel line pass: its 8192-point twiddles tw_lx (tw_x below
@@ -252,7 +252,7 @@ void free_plan(cwo_plan* p) {
     cudaFree(p->fpre_x); cudaFree(p->fpre_y); cudaFree(p->fpost_x); cudaFree(p->fpost_y);
     cudaFree(p->fst_x); cudaFree(p->frow_y);
     cudaFree(p->fpre_cx); cudaFree(p->fpre_cy); cudaFree(p->fpost_cx); cudaFree(p->fpost_cy);
-    cudaFree(p->hcache); cudaFree(p->hshared);
+    cudaFree(p->hcache);
     cudaFree(p->split_tw);
     cudaFree(p->hxl); cudaFree(p->zhxl);
     delete p;
@@ -319,7 +319,7 @@ cwo_status ensure_scratch(cwo_plan* p, int items) {
     cudaFree(p->scratch);
     p->scratch = nullptr;
     p->scap = 0;
-    cwo_status st = dev_alloc(&p->scratch, (size_t)items * p->ny * p->px, "scratch");
+    cwo_status st = dev_alloc(&p->scratch, scratch_entries(p->ny, p->px, items), "scratch");
     if (st != CWO_OK) return st;
     // wmap_s for every type: the mixed batches of any plan run their Fresnel items as line passes
     if ((e = cwo::make_intermediate_map(&p->wmap_f, p->scratch, p->ny, p->px, items, cwo::row_block_rows(p->px, false))) ||
@@ -328,11 +328,6 @@ cwo_status ensure_scratch(cwo_plan* p, int items) {
          (e = cwo::make_intermediate_map(&p->wmap_s, p->scratch, p->ny, p->nx, items, cwo::line_block_rows(p->px)))))
         return cuda_fail(e, "tensor map of the intermediate");
     p->scap = items;
-    if (p->type == CWO_ANGULAR && !p->hshared && !p->hcache && p->flags == 0 && shared_h_entries(p->nx, p->ny, items) &&
-        cudaMalloc((void**)&p->hshared, shared_h_entries(p->nx, p->ny, items) * sizeof(float2)) != cudaSuccess) {
-        cudaGetLastError();
-        p->hshared = nullptr;   // without it the call runs as before
-    }
     return CWO_OK;
 }
 
@@ -523,8 +518,13 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
         if (epi.mode == cwo::EPI_INTENSITY && (st = check_device_range(epi.inten, rb, p->device, "intensity"))) return st;
     }
     }
-    const int need = stack ? batch + 1 : batch;
-    if ((st = ensure_scratch(p, need))) return st;
+    // one transfer function for the whole batch, in the scratch of one more field: taken if that is there (by
+    // cwo_plan_reserve), asked for if the scratch grows anyway
+    const bool share = !zs && !stack && p->type == CWO_ANGULAR && p->flags == 0 && shared_h_worth(p->nx, p->ny, batch) &&
+                       asm_tail_mode(p->px, p->py, p->dx, p->dy, p->lambda, p->z) < 2;   // not where the phase needs FP64
+    if (!(share && p->scap < batch && ensure_scratch(p, batch + 1) == CWO_OK) &&
+        (st = ensure_scratch(p, stack ? batch + 1 : batch)))
+        return st;
 
     cudaStream_t s = (cudaStream_t)stream;
     if (p->type == CWO_FRESNEL_FOURIER) {
@@ -598,12 +598,12 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
             hp.hcache_stride = p->py;
             hp.split_tw = p->split_tw;
             hp.split_w = p->split_w;
-        } else if (p->hshared && !stack && shared_h_entries(p->nx, p->ny, batch) &&
-                   (hp.mode == cwo::HMODE_ASM_POLY || hp.mode == cwo::HMODE_ASM_EXACT)) {
-            const cudaError_t e = cwo::launch_build_hcache(p->hshared, hp.npairs, p->py, hp, s);
+        } else if (share && p->scap > batch) {
+            float2* table = p->scratch + (size_t)batch * p->ny * p->px;
+            const cudaError_t e = cwo::launch_build_hcache(table, hp.npairs, p->py, hp, s);
             if (e != cudaSuccess) return cuda_fail(e, "transfer-function launch");
             hp.mode = cwo::HMODE_TABLE;
-            hp.hcache = p->hshared;
+            hp.hcache = table;
             hp.hcache_stride = p->py;
         }
     }
@@ -1065,7 +1065,7 @@ cwo_status cwo_plan_device_bytes(int nx, int ny, int batch, size_t* bytes) {
     if (!bytes) return fail(CWO_ERR_INVALID_ARG, "bytes is NULL");
     if (!pow2_side(nx) || !pow2_side(ny)) return fail(CWO_ERR_INVALID_ARG, "Nx=%d, Ny=%d out of range", nx, ny);
     if (batch < 1) return fail(CWO_ERR_INVALID_ARG, "batch must be >= 1");
-    *bytes = tables_bytes(nx, ny) + shared_h_entries(nx, ny, batch) * sizeof(float2) + (size_t)batch * ny * (2 * (size_t)nx) * sizeof(float2) +
+    *bytes = tables_bytes(nx, ny) + scratch_entries(ny, 2 * nx, batch) * sizeof(float2) +
              (size_t)batch * (2 * (size_t)nx + 2 * (size_t)ny) * sizeof(float4) + (size_t)batch * sizeof(cwo::ItemParams);
     return CWO_OK;
 }
