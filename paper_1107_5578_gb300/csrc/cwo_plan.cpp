@@ -1197,11 +1197,16 @@ cwo_status cwo_propagate_rows(cwo_plan* p, const void* in_c64, void* out_c64, in
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const long long field = (long long)p->nx * p->ny, wstride = (long long)p->ny * p->px;
     const float scale = (float)(1.0 / ((double)p->px * (double)p->py));
-    if ((e = cwo::launch_row_fwd(p->px, (const float2*)in_c64 + (size_t)hp.ylo * p->nx, field, &mf, 0, hp.yhi - hp.ylo, 1, p->tw_x, p->status, s)))
+    const bool timing = p->tev[0] != nullptr;
+    auto mark = [&](int i) { return timing ? cudaEventRecord(p->tev[i], s) : cudaSuccess; };
+    if ((e = mark(0)) ||
+        (e = cwo::launch_row_fwd(p->px, (const float2*)in_c64 + (size_t)hp.ylo * p->nx, field, &mf, 0, hp.yhi - hp.ylo, 1, p->tw_x, p->status, s)) ||
+        (e = mark(1)))
         return cuda_fail(e, "row forward launch");
-    if ((e = cwo::launch_col(p->py, p->scratch, wstride, p->scratch, wstride, p->px, 1, p->tw_y, hp, s)))
+    if ((e = cwo::launch_col(p->py, p->scratch, wstride, p->scratch, wstride, p->px, 1, p->tw_y, hp, s)) || (e = mark(2)))
         return cuda_fail(e, "column launch");
-    if ((e = cwo::launch_row_inv(p->px, &mi, 0, (float2*)out_c64 + (size_t)hp.olo * p->nx, field, hp.ohi - hp.olo, 1, scale, p->tw_x, p->status, s)))
+    if ((e = cwo::launch_row_inv(p->px, &mi, 0, (float2*)out_c64 + (size_t)hp.olo * p->nx, field, hp.ohi - hp.olo, 1, scale, p->tw_x, p->status, s)) ||
+        (e = mark(3)))
         return cuda_fail(e, "row inverse launch");
     return CWO_OK;
 }
