@@ -316,9 +316,10 @@ cwo_status cwo_plan_check(cwo_plan* plan);
 
 /* Instrumentation: when `events` is non-NULL it must point to 4 cudaEvent_t (passed as void*)
  * created by the caller on the plan's device; every later call records events[0] before the row
- * forward pass, events[1] after it, events[2] after the column pass and events[3] after the row
- * inverse pass, on the call's stream, so that per-pass durations can be read with
- * cudaEventElapsedTime.  NULL switches recording off.  The caller keeps ownership of the events. */
+ * forward pass, events[1] after it, events[2] after the column pass (with the transfer function of a
+ * large batch of small fields, evaluated just before it) and events[3] after the row inverse pass, on
+ * the call's stream, so that per-pass durations can be read with cudaEventElapsedTime.  NULL switches
+ * recording off.  The caller keeps ownership of the events. */
 cwo_status cwo_plan_set_timing_events(cwo_plan* plan, void* const* events);
 
 /*

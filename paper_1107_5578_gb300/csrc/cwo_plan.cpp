@@ -598,13 +598,6 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
             hp.hcache_stride = p->py;
             hp.split_tw = p->split_tw;
             hp.split_w = p->split_w;
-        } else if (share && p->scap > batch) {
-            float2* table = p->scratch + (size_t)batch * p->ny * p->px;
-            const cudaError_t e = cwo::launch_build_hcache(table, hp.npairs, p->py, hp, s);
-            if (e != cudaSuccess) return cuda_fail(e, "transfer-function launch");
-            hp.mode = cwo::HMODE_TABLE;
-            hp.hcache = table;
-            hp.hcache_stride = p->py;
         }
     }
 
@@ -697,8 +690,16 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
                     return cuda_fail(e, "column launch");
             }
             if ((e = mark(2))) return cuda_fail(e, "event");
-        } else if ((e = cwo::launch_col(p->py, p->scratch, wstride, p->scratch, wstride, p->px, batch, p->tw_y, hp, s)) || (e = mark(2))) {
-            return cuda_fail(e, "column launch");
+        } else {
+            if (share && p->scap > batch) {
+                float2* table = p->scratch + batch * wstride;
+                if ((e = cwo::launch_build_hcache(table, hp.npairs, p->py, hp, s))) return cuda_fail(e, "transfer-function launch");
+                hp.mode = cwo::HMODE_TABLE;
+                hp.hcache = table;
+                hp.hcache_stride = p->py;
+            }
+            if ((e = cwo::launch_col(p->py, p->scratch, wstride, p->scratch, wstride, p->px, batch, p->tw_y, hp, s)) || (e = mark(2)))
+                return cuda_fail(e, "column launch");
         }
         if ((e = cwo::launch_row_inv(p->px, &p->wmap_i, 0, fout, field, p->ny, batch, scale, p->tw_x, p->status, s, ep)) ||
             (e = mark(3)))
