@@ -301,13 +301,18 @@ cwo_status cwo_hologram_forward(cwo_plan* plan, const float* phase, const float*
 cwo_status cwo_hologram_backward(cwo_plan* plan, const float* phase, const void* u_c64, const float* g, const float* gloss,
                                  int h, int w, int ox, int oy, void* work_c64, float* gphase, void* cuda_stream);
 
-/* Number of kernel launches one call of cwo_propagate_batch makes for this plan (for launch
- * accounting in benchmarks): 3 for the angular spectrum types (one more for a large batch of small
- * fields, whose transfer function is evaluated once for all of them), 2 for the Fresnel Fourier form and
- * for the Fresnel convolution and shifted Fresnel types, whose separable line passes take 2 (3
- * for an output epilogue, an output or a stack source not on a 16-byte boundary, a shifted
- * Fresnel z-stack, or a z-stack of padded rows longer than 4096). */
+/* Number of kernel launches one call of cwo_propagate makes for this plan (for launch accounting in
+ * benchmarks), which is also the number of passes of every batched call: 3 for the angular spectrum types,
+ * 2 for the Fresnel Fourier form and for the Fresnel convolution and shifted Fresnel types, whose
+ * separable line passes take 2 (3 for an output epilogue, an output or a stack source not on a 16-byte
+ * boundary, a shifted Fresnel z-stack, or a z-stack of padded rows longer than 4096). */
 int cwo_launches_per_call(const cwo_plan* plan);
+
+/* The launches of the next cwo_propagate_batch with one input per field and these distances: the passes above
+ * and, for CWO_ANGULAR, what evaluates the transfer function beside them: one launch for a large batch of small
+ * fields at the plan's distance, one per 24 distances that differ from the last call's, or one
+ * column pass per field where a distance needs the phase in FP64.  0 for a NULL plan or batch < 1. */
+int cwo_launches_per_batch(const cwo_plan* plan, int batch, const double* z_or_null);
 
 /* Synchronise the device and report whether any earlier call on this plan had a bounded wait
  * expire (CWO_ERR_TIMEOUT; the affected outputs were not written).  The waits guard asynchronous

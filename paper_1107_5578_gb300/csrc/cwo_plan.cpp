@@ -472,6 +472,17 @@ cwo_status asm_tables(const cwo_plan* p, int items, const Params& params, const 
     return CWO_OK;
 }
 
+// the per-item buffers hold the tables of these distances
+bool holds_tables(const cwo_plan* p, const double* zs, int batch) {
+    return (int)p->zs_cached.size() == batch && std::equal(p->zs_cached.begin(), p->zs_cached.end(), zs);
+}
+
+// a batch at the plan's distance evaluates its transfer function once (not where the phase needs FP64)
+bool shares_h(const cwo_plan* p, int batch) {
+    return p->type == CWO_ANGULAR && p->flags == 0 && shared_h_worth(p->nx, p->ny, batch) &&
+           asm_tail_mode(p->px, p->py, p->dx, p->dy, p->lambda, p->z) < 2;
+}
+
 // prevalidated: the caller (one API call that propagates the same buffers repeatedly) has
 // already checked these buffers with this plan
 cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int batch,
@@ -520,8 +531,7 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
     }
     // one transfer function for the whole batch, in the scratch of one more field: taken if that is there (by
     // cwo_plan_reserve), asked for if the scratch grows anyway
-    const bool share = !zs && !stack && p->type == CWO_ANGULAR && p->flags == 0 && shared_h_worth(p->nx, p->ny, batch) &&
-                       asm_tail_mode(p->px, p->py, p->dx, p->dy, p->lambda, p->z) < 2;   // not where the phase needs FP64
+    const bool share = !zs && !stack && shares_h(p, batch);
     if (!(share && p->scap < batch && ensure_scratch(p, batch + 1) == CWO_OK) &&
         (st = ensure_scratch(p, stack ? batch + 1 : batch)))
         return st;
@@ -549,8 +559,7 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
     const bool per_item_k = zs && hp.mode == cwo::HMODE_ASM_FP64;
 
     // per-item tables of the same distances as the previous call are reused ("once-calculation")
-    const bool ztables_hit = zs && !per_item_k && (int)p->zs_cached.size() == batch &&
-                             std::equal(p->zs_cached.begin(), p->zs_cached.end(), zs);
+    const bool ztables_hit = zs && !per_item_k && holds_tables(p, zs, batch);
     if (zs && !per_item_k && ztables_hit) {
         if (p->type == CWO_ANGULAR) {
             hp.ax = p->zax; hp.ay = p->zay; hp.kf = p->zkf;
@@ -1287,6 +1296,15 @@ cwo_status cwo_gs_run(cwo_plan* plan, const float* amplitude, void* field_c64, f
 int cwo_launches_per_call(const cwo_plan* plan) {
     if (!plan) return 0;
     return plan->type == CWO_FRESNEL_FOURIER || plan->type == CWO_FRESNEL_CONV || plan->type == CWO_SHIFTED_FRESNEL ? 2 : 3;
+}
+
+int cwo_launches_per_batch(const cwo_plan* plan, int batch, const double* z_or_null) {
+    if (!plan || batch < 1) return 0;
+    const int passes = cwo_launches_per_call(plan);
+    if (plan->type != CWO_ANGULAR) return passes;
+    if (!z_or_null) return passes + (shares_h(plan, batch) && plan->scap != batch);
+    if (base_hparams(plan, z_or_null, batch).mode == cwo::HMODE_ASM_FP64) return passes - 1 + batch;
+    return passes + (holds_tables(plan, z_or_null, batch) ? 0 : (batch + cwo::kAsmItems - 1) / cwo::kAsmItems);
 }
 
 cwo_status cwo_plan_check(cwo_plan* plan) {

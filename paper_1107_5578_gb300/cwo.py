@@ -112,6 +112,7 @@ def lib() -> ctypes.CDLL:
                 "cwo_propagate_adjoint_batch": ([vp, vp, ll, vp, i, dpp, vp], i),
                 "cwo_propagate_items": ([vp, vp, ll, vp, i, ctypes.POINTER(Item), vp], i),
                 "cwo_launches_per_call": ([vp], i),
+                "cwo_launches_per_batch": ([vp, i, vp], i),
                 "cwo_propagate_epilogue": ([vp, vp, vp, i, i, i, vp, vp, vp], i),
                 "cwo_gs_run": ([vp, vp, vp, vp, i, i, vp], i),
                 "cwo_hologram_forward": ([vp, vp, vp, i, i, i, i, vp, vp, vp, vp, vp], i),
@@ -291,6 +292,13 @@ class Plan:
     @property
     def launches_per_call(self) -> int:
         return int(lib().cwo_launches_per_call(self.handle))
+
+    def launches_per_batch(self, batch: int, z=None) -> int:
+        """Kernel launches of the next propagate_batch of ``batch`` fields (at the distances ``z``)."""
+        if z is not None and len(z) != batch:
+            raise ValueError(f"{len(z)} distances for {batch} items")
+        zp = None if z is None else (ctypes.c_double * batch)(*map(float, z))
+        return int(lib().cwo_launches_per_batch(self.handle, int(batch), zp))
 
     def _out(self, x, batch_shape):
         torch = _torch or _load_torch()
