@@ -45,6 +45,12 @@ class _Geometry:
 
     def backward(self, phi, u, g, gloss):
         """derivative by the phase, through the adjoint kernels"""
+        h, w = self.window[:2]
+        if phi.shape != (h, w) or g.shape != (h, w) or u.shape != (self.canvas, self.canvas):
+            raise RuntimeError("a saved tensor came back with another shape")
+        # saved-tensor hooks may hand back another type than they were given
+        if not phi.dtype == g.dtype == torch.float32 or u.dtype != torch.complex64:
+            phi, u, g = phi.float(), u.to(torch.complex64), g.float()
         phi, u, g = phi.contiguous(), u.contiguous(), g.contiguous()
         work, out = torch.empty_like(u), torch.empty_like(phi)
         _call("cwo_hologram_backward", self.plan.handle, phi.data_ptr(), u.data_ptr(), g.data_ptr(),
