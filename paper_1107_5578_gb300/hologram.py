@@ -149,7 +149,7 @@ class HologramProblem:
 
     def _own(self, step: str) -> bool:
         """the step is the one below, replaced neither by a subclass nor in the instance or the class"""
-        return getattr(getattr(self, step), "__func__", None) is _STEPS[step]
+        return getattr(type(self), step) is _STEPS[step] and step not in self.__dict__
 
     def _fused(self, phi) -> bool:
         return self._own("field") and self._window(phi) and self.plan.nx == self.plan.ny == self.canvas \
