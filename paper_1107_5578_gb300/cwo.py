@@ -77,6 +77,19 @@ def _int32(v: int) -> int:
     return (v + (1 << 31)) % (1 << 32) - (1 << 31)
 
 
+def item_records(items):
+    """The records of a mixed batch (an array of Item) from dicts, Item structures or ones derived from it."""
+    buf = bytearray(len(items) * _ITEM.size)
+    for k, it in enumerate(items):
+        if isinstance(it, Item):
+            buf[k * _ITEM.size:(k + 1) * _ITEM.size] = bytes(it)[:_ITEM.size]   # without a derived one's own fields
+        else:
+            _ITEM.pack_into(buf, k * _ITEM.size, float(it["z"]), float(it["wavelength"]), float(it["dx"]),
+                            float(it.get("dy", it["dx"])), _int32(int(it["type"])),
+                            int(it.get("flags", 0)) & 0xFFFFFFFF)
+    return (Item * len(items)).from_buffer(buf)
+
+
 class CwoError(RuntimeError):
     def __init__(self, status: int, where: str, message: str):
         self.status = status
@@ -357,15 +370,7 @@ class Plan:
         _check_field(x, self.nx, self.ny, "input", b)
         if len(items) != b:
             raise ValueError(f"{len(items)} items for {b} fields")
-        buf = bytearray(b * ctypes.sizeof(Item))
-        for k, it in enumerate(items):
-            if isinstance(it, Item):
-                buf[k * _ITEM.size:(k + 1) * _ITEM.size] = bytes(it)
-            else:
-                _ITEM.pack_into(buf, k * _ITEM.size, float(it["z"]), float(it["wavelength"]), float(it["dx"]),
-                                float(it.get("dy", it["dx"])), _int32(int(it["type"])),
-                                int(it.get("flags", 0)) & 0xFFFFFFFF)
-        arr = (Item * b).from_buffer(buf)
+        arr = item_records(items)
         out = self._result(x, out, (b,), b)
         check(lib().cwo_propagate_items(self.handle, x.data_ptr(), self.nx * self.ny, out.data_ptr(), b, arr,
                                         _stream_handle(stream)), "cwo_propagate_items")
