@@ -323,16 +323,20 @@ static cudaError_t col_impl_t(const float2* win, long long win_item_stride, floa
         if (e != cudaSuccess) return e;
     } else {         // H even in kx: mirror pairs
         if (hp.npairs != px / 2 + 1 || !hp.pairs) return cudaErrorInvalidValue;
-        // two pairs per CTA at P = 2048 for a batch that evaluates H per element: the CTA's pairs share the
-        // item's y table in L1 (7 1024^2 fields with their own distances 112.4 us against 114.2 for one
-        // pair; cached, 16 fields, 219 against 216)
+        // Two pairs per CTA at P = 2048 where H is evaluated by its series and the pairs fill the chip (152 SMs x 8)
+        // about three times: the CTA's pairs share the item's y table in L1.  Whole calls, one and two pairs, us:
+        // 7 512 x 1024 fields 97.0 and 95.1, 7 1024^2 188.9 and 187.8, 16 411.7 and 408.5, 7 2048 x 1024 385.0 and
+        // 382.9; but with fewer pairs the last wave decides: 12 256 x 1024 fields (3084 pairs) 80.8 and 82.4, 4
+        // 30.5 and 33.1.  Not in the closed form (7 1024^2 fields 212.2 and 216.7).  A mixed batch takes one
+        // pair whatever its items, so that an item runs the same kernel alone and in company (7 1024^2
+        // items by the series 196.4 and 194.7, in closed form 217.9 and 222.6).
         constexpr int CP = cols_per_block<P>();
         if constexpr (!MIXED) {
             if (hp.win) return colp_launch<P, CP, false, true>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);
         }
-        if constexpr (P == 2048) {
-            if (hp.mode != HMODE_TABLE && items >= 4)
-                return colp_launch<P, 2 * CP, MIXED>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);
+        if constexpr (P == 2048 && !MIXED) {
+            if (hp.mode == HMODE_ASM_POLY && items >= 4 && (long long)items * hp.npairs >= 3500)
+                return colp_launch<P, 2 * CP, false>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);
         }
         return colp_launch<P, CP, MIXED>(win, win_item_stride, wout, wout_item_stride, items, tw, hp, st);
     }
