@@ -405,7 +405,7 @@ k_row_inv_p(const __grid_constant__ CUtensorMap wmap, int item_off, float2* __re
     }
 }
 
-// Turn (P <= 4096): the inverse row pass of one propagation and the forward row pass of the next
+// Turn (P <= 2048): the inverse row pass of one propagation and the forward row pass of the next
 // in one kernel, for loops that constrain the field between propagations (the GS iteration of
 // Section "GS algorithm").  A CTA loads its R rows of the intermediate by TMA, takes their
 // inverse FFTs, crops to the Nx kept samples, scales, applies the constraint (EPI_PHASE or
@@ -414,7 +414,8 @@ k_row_inv_p(const __grid_constant__ CUtensorMap wmap, int item_off, float2* __re
 // ends with register e of thread t at position t + e T, which is where the forward's first
 // stage takes its inputs, so the crop, constraint and padding act on the registers and no
 // exchange is added; each row's arithmetic is that of k_row_inv_p followed by k_row_fwd_p, so
-// the loop computes bit for bit what the separate passes compute through the stored field.
+// the loop computes bit for bit what the separate passes compute through the stored field (not at
+// P = 4096, where k_row_inv_p merges its roots).
 template <int P, int R, int EPI>
 __global__ void __launch_bounds__(R * (P / 16))
 k_row_turn(const __grid_constant__ CUtensorMap wmap, int groups_per_item, long long field_item_stride,
@@ -465,19 +466,16 @@ k_row_turn(const __grid_constant__ CUtensorMap wmap, int groups_per_item, long l
 template <int P, int EPI>
 static cudaError_t row_turn_impl(const CUtensorMap* wmap, int ny, int items, long long field_item_stride, float scale,
                                  const float4* tw, int* status, const Epilogue& ep, cudaStream_t st) {
-    if constexpr (P > 4096 || P < 64) {
-        return cudaErrorNotSupported;
-    } else {
-        constexpr int R = rows_fwd<P>();
-        constexpr int T = P / 16;
-        if (ny % R || items < 1 || !status) return cudaErrorInvalidValue;
-        const size_t smem = row_smem_words<P, R>() * sizeof(float2) + sizeof(uint64_t);
-        cudaError_t e = kernel_setup<k_row_turn<P, R, EPI>>(smem, R * T, nullptr);
-        if (e != cudaSuccess) return e;
-        const int groups = ny / R;
-        return pdl_launch(k_row_turn<P, R, EPI>, dim3((unsigned)(groups * items)), dim3(R * T), smem, st, *wmap, groups,
-                          field_item_stride, scale, tw, status, ep);
-    }
+    static_assert(P >= 64 && P <= 2048, "row_turn_supported");
+    constexpr int R = rows_fwd<P>();
+    constexpr int T = P / 16;
+    if (ny % R || items < 1 || !status) return cudaErrorInvalidValue;
+    const size_t smem = row_smem_words<P, R>() * sizeof(float2) + sizeof(uint64_t);
+    cudaError_t e = kernel_setup<k_row_turn<P, R, EPI>>(smem, R * T, nullptr);
+    if (e != cudaSuccess) return e;
+    const int groups = ny / R;
+    return pdl_launch(k_row_turn<P, R, EPI>, dim3((unsigned)(groups * items)), dim3(R * T), smem, st, *wmap, groups,
+                      field_item_stride, scale, tw, status, ep);
 }
 
 template <int P, bool PRE>

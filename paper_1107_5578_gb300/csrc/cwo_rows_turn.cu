@@ -15,7 +15,7 @@ cudaError_t launch_row_turn(int px, const CUtensorMap* wmap, int ny, int items, 
 #define CASE(P) case P: return ep.mode == EPI_PHASE \
         ? row_turn_impl<P, EPI_PHASE>(wmap, ny, items, field_item_stride, scale, tw, status, ep, st) \
         : row_turn_impl<P, EPI_AMPLITUDE>(wmap, ny, items, field_item_stride, scale, tw, status, ep, st);
-        CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024) CASE(2048) CASE(4096)
+        CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024) CASE(2048)
 #undef CASE
         default: return cudaErrorNotSupported;
     }
