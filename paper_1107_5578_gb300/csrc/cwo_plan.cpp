@@ -192,6 +192,7 @@ struct cwo_plan {
     float* zkf = nullptr;
     StagingRing zstage;   // pinned staging of the per-item z tables
     std::vector<double> zs_cached;   // distances whose tables the per-item buffers hold
+    bool zs_captured = false;        // a graph holds launches that write these buffers: nothing is known of them
     // mixed-batch (cwo_propagate_items) per-item tables and parameters
     int icap = 0;
     float4* ix = nullptr; float4* iy = nullptr; cwo::ItemParams* iprm = nullptr;
@@ -559,6 +560,13 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
     const bool per_item_k = zs && hp.mode == cwo::HMODE_ASM_FP64;
 
     // per-item tables of the same distances as the previous call are reused ("once-calculation")
+    if (zs && !per_item_k && !p->zs_captured) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing");
+        p->zs_captured = cap != cudaStreamCaptureStatusNone;
+        if (p->zs_captured) p->zs_cached.clear();
+    }
     const bool ztables_hit = zs && !per_item_k && holds_tables(p, zs, batch);
     if (zs && !per_item_k && ztables_hit) {
         if (p->type == CWO_ANGULAR) {
@@ -597,7 +605,7 @@ cwo_status run(cwo_plan* p, const void* in, long long in_stride, void* out, int 
             hp.x_item_stride = p->px; hp.y_item_stride = p->py;
             if ((st = staging_release_after(p->zstage, zslot, s))) return st;
         }
-        p->zs_cached.assign(zs, zs + batch);
+        if (!p->zs_captured) p->zs_cached.assign(zs, zs + batch);
     } else {
         hp.ax = p->ax; hp.ay = p->ay; hp.kf = p->kf; hp.hx = p->hx; hp.hy = p->hy;
         hp.x_item_stride = 0; hp.y_item_stride = 0; hp.kf_item_stride = 0;
