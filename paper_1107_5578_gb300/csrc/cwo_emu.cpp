@@ -42,7 +42,8 @@ void emu_exchange(std::vector<Regs>& R) {
         for (int e = 0; e < 16; ++e) R[t].v[e] = sm[PadLayout<P, 1>::addr(0, stage_pos<P, SR>(t, e))];
 }
 
-// MERGED as in the kernels: the plain columns and lines of P = 4096 (not the split column pass)
+// MERGED as in the pair kernels: columns and lines of P = 4096 (not the split column pass; the forward row pass at
+// 4096 keeps the plain form, and the single-column kernel merges at 2048 too: the same DFT up to rounding)
 template <int P, int S, int NZ0, bool MERGED = P == 4096>
 void emu_fwd_from(std::vector<Regs>& R, const float4* tw) {
     using G = Geo<P>;

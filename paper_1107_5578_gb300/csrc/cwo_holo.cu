@@ -5,7 +5,7 @@
 // All five are elementwise over the canvas or the window and bound by memory: each reads what it needs
 // once and writes its result once, two complex values a thread.  As separate tensor operators a
 // loss and its gradient at 1080 x 1920 in a 2048^2 canvas were about 60 launches and 960 us of host
-// time around 250 us of propagation; now 12 launches from two calls, and the propagations leave out the
+// time around 250 us of propagation; now 11 launches from two calls, and the propagations leave out the
 // canvas rows outside the window (125 -> 99 us each): 260 us in all.  The window may start at any column and have any width: the
 // canvas is walked in 16-byte pairs and each of the pair's pixels is tested.
 #include <cuda_runtime.h>
