@@ -21,13 +21,18 @@ import torch
 from . import autograd, cwo, synth
 
 
+_F32, _C64 = torch.float32, torch.complex64
+
+
 class _Geometry:
     """The window of a problem on its canvas and the plan that propagates it, as they were at the call."""
-    __slots__ = ("plan", "window", "canvas")
+    __slots__ = ("plan", "window", "canvas", "shapes")
 
     def __init__(self, p: "HologramProblem"):
         self.plan, self.canvas = p.plan, p.canvas
-        self.window = (p.h, p.w, p.ox, p.oy)
+        h, w = p.h, p.w
+        self.window = (h, w, p.ox, p.oy)
+        self.shapes = ((h, w), (h, w), (p.canvas, p.canvas))   # of phase, gradient and field
 
     def forward(self, phi, target):
         """(u, |u|^2) of u = A exp(i phi), or, with a target, (u, residual, loss)"""
@@ -45,12 +50,11 @@ class _Geometry:
 
     def backward(self, phi, u, g, gloss):
         """derivative by the phase, through the adjoint kernels"""
-        h, w = self.window[:2]
-        if phi.shape != (h, w) or g.shape != (h, w) or u.shape != (self.canvas, self.canvas):
-            raise RuntimeError("a saved tensor came back with another shape")
         # saved-tensor hooks may hand back another type than they were given
-        if not phi.dtype == g.dtype == torch.float32 or u.dtype != torch.complex64:
-            phi, u, g = phi.float(), u.to(torch.complex64), g.float()
+        if phi.dtype is not _F32 or g.dtype is not _F32 or u.dtype is not _C64:
+            phi, u, g = phi.float(), u.to(_C64), g.float()
+        if (phi.shape, g.shape, u.shape) != self.shapes:
+            raise RuntimeError("a saved tensor came back with another shape")
         phi, u, g = phi.contiguous(), u.contiguous(), g.contiguous()
         work, out = torch.empty_like(u), torch.empty_like(phi)
         _call("cwo_hologram_backward", self.plan.handle, phi.data_ptr(), u.data_ptr(), g.data_ptr(),
@@ -147,12 +151,10 @@ class HologramProblem:
         return type(t) in (torch.Tensor, torch.nn.Parameter) and t.dtype == torch.float32 and t.is_cuda \
             and t.shape == (self.h, self.w) and not t.is_neg()
 
-    def _own(self, step: str) -> bool:
-        """the step is the one below, replaced neither by a subclass nor in the instance or the class"""
-        return getattr(type(self), step) is _STEPS[step] and step not in self.__dict__
-
+    # a step that a subclass, the instance or a patch of this class has replaced is called: the fused kernels do the
+    # work of the ones below only
     def _fused(self, phi) -> bool:
-        return self._own("field") and self._window(phi) and self.plan.nx == self.plan.ny == self.canvas \
+        return getattr(self.field, "__func__", None) is _FIELD and self._window(phi) and self.plan.nx == self.plan.ny == self.canvas \
             and 0 <= self.oy <= self.canvas - self.h and 0 <= self.ox <= self.canvas - self.w
 
     def intensity(self, phi: torch.Tensor) -> torch.Tensor:
@@ -161,13 +163,13 @@ class HologramProblem:
 
     def loss(self, phi: torch.Tensor) -> torch.Tensor:
         geo, t = _Geometry(self), self.target
-        if self._own("intensity") and self._fused(phi) and self._window(t) and t.is_contiguous() and not t.requires_grad and t.device == phi.device:
+        if getattr(self.intensity, "__func__", None) is _INTENSITY and self._fused(phi) and self._window(t) and t.is_contiguous() and not t.requires_grad and t.device == phi.device:
             return _Loss.apply(phi, t, geo)
         d = self.intensity(phi) - t
         return (d * d).mean()
 
 
-_STEPS = {"field": HologramProblem.field, "intensity": HologramProblem.intensity}
+_FIELD, _INTENSITY = HologramProblem.field, HologramProblem.intensity
 
 
 def optimise(problem: HologramProblem, steps=200, lr=0.05, log_every=0):
